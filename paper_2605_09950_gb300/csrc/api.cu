@@ -358,8 +358,16 @@ static int session_init(boruta_session* s, const uint8_t* X, int64_t ld, const v
     if ((rc = s->alloc(&d.nd_cnt, P * d.C))) return rc;
     if ((rc = s->alloc(&d.nd_lcnt, P * d.C))) return rc;
   }
-  // larger nodes of one level: at most N/33 per tree (each has > 32 rows)
-  const size_t big_cap = static_cast<size_t>(n_trees) * (static_cast<size_t>(N) / 33 + 1);
+  // larger nodes of one level: at most N/33 per tree (each has > 32 rows), or
+  // N/65 for classification (> 64 rows; mid nodes: N/33 of > 32 rows, and N/67
+  // of weight > 66)
+  const size_t big_rows = reg ? kFewRows : kMidRows;
+  const size_t big_cap = static_cast<size_t>(n_trees) * (static_cast<size_t>(N) / (big_rows + 1) + 1);
+  if (!reg) {
+    const size_t mid_cap = static_cast<size_t>(N) / (kFewRows + 1) + static_cast<size_t>(N) / (kFewWeight + 1) + 2;
+    if ((rc = s->alloc(&d.mid, static_cast<size_t>(n_trees) * mid_cap))) return rc;
+    if ((rc = s->alloc(&d.nmid, max_depth + 2))) return rc;
+  }
   if ((rc = s->alloc(&d.big, big_cap))) return rc;
   uint8_t* ninfo = nullptr;
   if ((rc = s->alloc(&ninfo, big_cap * ninfo_bytes(split_variant(d.kind, d.C))))) return rc;
@@ -549,6 +557,7 @@ static int enqueue_iteration(boruta_session* s, int t, cudaStream_t st) {
   CK(cudaMemsetAsync(d.nsmall, 0, (d.D + 2) * sizeof(uint32_t), st));
   CK(cudaMemsetAsync(d.ntiny, 0, (d.D + 2) * sizeof(uint32_t), st));
   CK(cudaMemsetAsync(d.nmicro, 0, (d.D + 2) * sizeof(uint32_t), st));
+  if (d.nmid) CK(cudaMemsetAsync(d.nmid, 0, (d.D + 2) * sizeof(uint32_t), st));
   CK(cudaMemsetAsync(d.lvl_cnt, 0, (d.D + 2) * sizeof(uint32_t), st));
   CK(cudaMemsetAsync(d.counters, 0, 4 * sizeof(unsigned long long), st));
 
@@ -570,10 +579,12 @@ static int enqueue_iteration(boruta_session* s, int t, cudaStream_t st) {
   for (int level = 0; level < d.D; ++level) {
     // grids sized to what the level can hold (every split kernel loops over
     // its work, so any grid is correct): at most M * min(2^level, N) nodes, of
-    // which at most M * min(2^level, N/33) have more than 32 rows
+    // which at most M * min(2^level, N/(r+1)) have more than r rows
     const uint64_t width = 1ull << level;
     const uint64_t nodes = static_cast<uint64_t>(d.M) * std::min<uint64_t>(width, static_cast<uint64_t>(d.N));
-    const uint64_t big = static_cast<uint64_t>(d.M) * std::min<uint64_t>(width, static_cast<uint64_t>(d.N) / 33);
+    const uint64_t big_rows = d.kind ? kFewRows : kMidRows;
+    const uint64_t big =
+        static_cast<uint64_t>(d.M) * std::min<uint64_t>(width, static_cast<uint64_t>(d.N) / (big_rows + 1));
     const uint64_t groups = big * static_cast<uint64_t>(d.mtry);  // work items of the larger nodes, at most
     const int gs = static_cast<int>(std::min<uint64_t>(s->small_grid, (nodes + 7) / 8));
     const int gi = static_cast<int>(std::min<uint64_t>(s->split_grid, std::max<uint64_t>(1, (groups + 7) / 8)));

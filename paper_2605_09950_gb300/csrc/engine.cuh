@@ -50,12 +50,15 @@ struct Dev {
   uint32_t *lvl_off, *lvl_cnt;   // [D + 2]
   uint32_t* work;                // [D + 2] per level: number of nodes in `big`
   uint32_t* chunk;               // [kScanBlocks] per-block split counts
-  uint32_t* big;                 // [big_cap] this level's active nodes with > 32 rows
+  uint32_t* big;                 // [big_cap] this level's active nodes of more rows than the lists below
   uint32_t* small;               // [level_cap] this level's active nodes with <= 32 rows
   uint32_t* nsmall;              // [D + 2] per level: number of 17..32-row nodes at the start of `small`
   uint32_t* ntiny;               // [D + 2] per level: number of 9..16-row nodes at the end of `small`
   uint32_t* micro;               // [small_cap] this level's active nodes with <= 8 rows
   uint32_t* nmicro;              // [D + 2] per level: number of them
+  uint32_t* mid;                 // [mid_cap] classification: nodes of 33..64 rows, and smaller ones
+                                 //   whose weight exceeds kFewWeight
+  uint32_t* nmid;                // [D + 2] per level: number of them
   uint32_t small_cap;            // entries of `small`
   void* ninfo;                   // [big_cap] node totals of `big`, by rank
   void* cand;                    // [big_cap * kItemsPerNode] best candidate per grouped item
@@ -90,6 +93,11 @@ struct Dev {
                                  // [3] node visits of the Alg. 3 tree walks
 };
 
+// Classification nodes of at most kFewRows rows and weight kFewWeight, and of
+// at most kMidRows rows of any weight, are split by matrix products
+// (small.cu); 66 is the largest weight whose terms n w (w <= 31) are exact in
+// half precision (at most 2048).
+constexpr uint32_t kFewRows = 32, kFewWeight = 66, kMidRows = 64;
 constexpr int kScanBlocks = 512;
 constexpr int kSplitThreads = 256;
 constexpr int kItemsPerNode = 16;  // work items (groups of draw slots) per larger node
@@ -118,6 +126,8 @@ int launch_bootstrap(const Dev& d, int grid, cudaStream_t st);
 int launch_split(const Dev& d, int level, int grid_small, int grid_big, uint64_t big_bound, size_t smem, cudaStream_t st,
                   cudaStream_t st2, cudaEvent_t fork, cudaEvent_t join, cudaEvent_t hist_start,
                   cudaEvent_t hist_end);
+// small.cu: the level's classification nodes of few rows, on `st`
+int launch_few_rows(const Dev& d, int level, int grid, cudaStream_t st);
 size_t ninfo_bytes(int variant);
 int split_variant(int kind, int C);
 int variant_classes(int variant);  // largest class count of a kernel variant (1 for regression)

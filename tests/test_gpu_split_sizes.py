@@ -1,0 +1,30 @@
+"""Split kernels at the sizes where their layouts change: nodes of 8, 16, 32
+and 64 rows (matrix-product split of few rows), samples around 32 features,
+2 to 8 classes, coarse bins (exact ties) and fine ones; every tree against
+the CPU oracle, bit for bit."""
+import numpy as np
+import pytest
+
+from paper_2605_09950_gb300 import synth
+from test_gpu_parity import built, check_iteration  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+def workload(N, p, classes, bins, n_trees, depth, mtry, seed, importance=synth.TREEIMP):
+    rng = np.random.default_rng(seed)
+    y = rng.integers(0, classes, size=N).astype(np.uint8)
+    y[:min(N, classes)] = np.arange(min(N, classes))
+    X = np.zeros((p, synth.pad16(N)), np.uint8)
+    X[:, :N] = rng.integers(0, bins, size=(p, N))
+    X[: p // 3, :N] = np.clip(X[: p // 3, :N] // 2 + y * (bins // (2 * classes)), 0, bins - 1)
+    return synth.Workload(f"N{N}", X, y, N, p, synth.CLASSIFICATION | importance, classes, bins, n_trees, depth, 2,
+                          seed=seed, mtry=mtry)
+
+
+@pytest.mark.parametrize("classes", [2, 3, 4, 5, 6, 8])
+@pytest.mark.parametrize("N,bins,mtry", [(13, 3, 31), (26, 256, 33), (51, 7, 40), (66, 256, 5), (104, 16, 33),
+                                         (410, 256, 32)])
+def test_small_nodes(classes, N, bins, mtry):
+    w = workload(N, 20, classes, bins, 24, 12, mtry, seed=N + classes)
+    check_iteration(w, tie_break=classes & 1)
