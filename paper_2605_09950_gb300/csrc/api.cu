@@ -97,6 +97,7 @@ struct boruta_session {
   // launch geometry
   int sms = 0, split_grid = 0, small_grid = 0, tree_grid = 0, permut_grid = 0, walk_grid = 0;
   size_t split_smem = 0;
+  int rec_grid[3] = {0, 0, 0};  // blocks of the three by-record kernels that the GPU holds at once
   // second stream for the small-node kernel, and its fork/join events
   cudaStream_t st2 = nullptr;
   cudaEvent_t fork = nullptr, join = nullptr;
@@ -367,6 +368,10 @@ static int session_init(boruta_session* s, const uint8_t* X, int64_t ld, const v
     const size_t mid_cap = static_cast<size_t>(N) / (kFewRows + 1) + static_cast<size_t>(N) / (kFewWeight + 1) + 2;
     if ((rc = s->alloc(&d.mid, static_cast<size_t>(n_trees) * mid_cap))) return rc;
     if ((rc = s->alloc(&d.nmid, max_depth + 2))) return rc;
+    if ((rc = s->alloc(&d.rec, static_cast<size_t>(n_trees) * (static_cast<size_t>(N) / (kMidRows + 1) + 1)))) return rc;
+    d.rec2_cap = static_cast<uint32_t>(n_trees) * (static_cast<uint32_t>(N) / 257u + 2u);
+    if ((rc = s->alloc(&d.rec2, d.rec2_cap))) return rc;
+    if ((rc = s->alloc(&d.nrec, 3 * (max_depth + 2)))) return rc;
   }
   if ((rc = s->alloc(&d.big, big_cap))) return rc;
   uint8_t* ninfo = nullptr;
@@ -434,6 +439,7 @@ static int session_init(boruta_session* s, const uint8_t* X, int64_t ld, const v
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kptr[1], kSplitThreads, s->split_smem));
   if (per_sm < 1) return fail(BORUTA_EINVAL, "split kernel does not fit on an SM");
   s->split_grid = per_sm * s->sms;
+  if (!reg) CK(static_cast<cudaError_t>(setup_record(variant, s->sms, s->rec_grid)));
   // warp-per-node kernels: as many blocks as the GPU holds at once (they
   // loop over their nodes), so no partial last wave
   int small_per_sm = 0;
@@ -482,6 +488,21 @@ int boruta_session_create(const uint8_t* X, int64_t ld, const void* y, int64_t N
   return 0;
 }
 
+// Largest classification node split by record (record.cu), 0 for none.  A
+// row's record costs about 20 sectors for 31 of 1000 columns, a column gather
+// one sector per row and column, fewer where a node holds more than one row in
+// 32.  Measured per level: with the row-major copy in L2 (N = 30011, 8
+// classes) records win at every size the tiles hold (10.2 -> 8.1 ms an
+// iteration); from DRAM the two cross at about N / 64 rows (N = 1e5, p = 1000:
+// 146.6 ms at N / 64, 151 at N / 32, 157 at N / 8, 164 without; N = 1e6: 955
+// against 1148 ms without, the same from N / 64 to N / 256).  Columns of at
+// most 4 bins stay with the register counts of the column path.
+static uint32_t record_rows(const boruta_session* s, const Dev& d) {
+  if (d.kind != 0 || s->split_path != 0 || d.B <= 4) return 0u;
+  const bool in_l2 = static_cast<uint64_t>(d.N) * static_cast<uint64_t>(d.ldP) <= (96ull << 20);
+  return std::min<uint32_t>(kRecordRows, static_cast<uint32_t>(d.N) / (in_l2 ? 1u : 64u));
+}
+
 // Enqueues iteration t on the session's stream (or records it, when the
 // stream is being captured into a graph), with the copies of its status,
 // state and counters into pinned host memory; does not wait.
@@ -502,6 +523,7 @@ static int enqueue_iteration(boruta_session* s, int t, cudaStream_t st) {
                               : (d.kind ? p_aug / 3 : isqrt(p_aug));
   d.mtry = static_cast<int32_t>(std::max<int64_t>(m, 1));
   d.ldP = static_cast<int32_t>((p_aug + 15) / 16 * 16);
+  d.rec_rows = record_rows(s, d);
   // feature bands: ~kBandBytes of columns each, at most kMaxBands; the packed
   // item holds a 14-bit slot and a 22-bit feature
   d.band_w = 0;
@@ -558,6 +580,7 @@ static int enqueue_iteration(boruta_session* s, int t, cudaStream_t st) {
   CK(cudaMemsetAsync(d.ntiny, 0, (d.D + 2) * sizeof(uint32_t), st));
   CK(cudaMemsetAsync(d.nmicro, 0, (d.D + 2) * sizeof(uint32_t), st));
   if (d.nmid) CK(cudaMemsetAsync(d.nmid, 0, (d.D + 2) * sizeof(uint32_t), st));
+  if (d.nrec) CK(cudaMemsetAsync(d.nrec, 0, 3 * (d.D + 2) * sizeof(uint32_t), st));
   CK(cudaMemsetAsync(d.lvl_cnt, 0, (d.D + 2) * sizeof(uint32_t), st));
   CK(cudaMemsetAsync(d.counters, 0, 4 * sizeof(unsigned long long), st));
 
@@ -597,7 +620,7 @@ static int enqueue_iteration(boruta_session* s, int t, cudaStream_t st) {
     }
     s->used_bw[level] = dl.band_w;
     s->used_bl[level] = dl.band_launch;
-    nk += launch_split(dl, level, std::max(gs, 1), gi, big, s->split_smem, st, s->st2, s->fork, s->join,
+    nk += launch_split(dl, level, std::max(gs, 1), gi, s->rec_grid, big, s->split_smem, st, s->st2, s->fork, s->join,
                        timed ? s->hev[2 * level] : nullptr, timed ? s->hev[2 * level + 1] : nullptr);
     CK_LAUNCH("split kernels");
     if (timed) CK(cudaEventRecord(s->ev[2 * level + 1], st));

@@ -59,6 +59,11 @@ struct Dev {
   uint32_t* mid;                 // [mid_cap] classification: nodes of 33..64 rows, and smaller ones
                                  //   whose weight exceeds kFewWeight
   uint32_t* nmid;                // [D + 2] per level: number of them
+  uint32_t* rec;                 // classification nodes split by record (record.cu): of 65..256 rows
+  uint32_t* rec2;                // [rec2_cap] of 257..1024 rows (from its start), of up to 4096 (from its end)
+  uint32_t* nrec;                // [D + 2][3] per level: numbers of the three
+  uint32_t rec2_cap;
+  uint32_t rec_rows;             // largest node split by record (0: none)
   uint32_t small_cap;            // entries of `small`
   void* ninfo;                   // [big_cap] node totals of `big`, by rank
   void* cand;                    // [big_cap * kItemsPerNode] best candidate per grouped item
@@ -98,6 +103,7 @@ struct Dev {
 // (small.cu); 66 is the largest weight whose terms n w (w <= 31) are exact in
 // half precision (at most 2048).
 constexpr uint32_t kFewRows = 32, kFewWeight = 66, kMidRows = 64;
+constexpr uint32_t kRecordRows = 4096;  // largest node of record.cu
 constexpr int kScanBlocks = 512;
 constexpr int kSplitThreads = 256;
 constexpr int kItemsPerNode = 16;  // work items (groups of draw slots) per larger node
@@ -123,11 +129,16 @@ int launch_bootstrap(const Dev& d, int grid, cudaStream_t st);
 // small-node kernel then runs on `st2` while the larger-node kernels run on
 // `st` (fork/join through the two events).
 // hist_start/hist_end are recorded on `st` around the histogram kernel.
-int launch_split(const Dev& d, int level, int grid_small, int grid_big, uint64_t big_bound, size_t smem, cudaStream_t st,
+int launch_split(const Dev& d, int level, int grid_small, int grid_big, const int* grid_rec, uint64_t big_bound,
+                  size_t smem, cudaStream_t st,
                   cudaStream_t st2, cudaEvent_t fork, cudaEvent_t join, cudaEvent_t hist_start,
                   cudaEvent_t hist_end);
 // small.cu: the level's classification nodes of few rows, on `st`
 int launch_few_rows(const Dev& d, int level, int grid, cudaStream_t st);
+// record.cu: shared memory limits and grid sizes of its three kernels; the
+// level's larger classification nodes of at most rec_rows rows, on `st`
+int setup_record(int variant, int sms, int* grids);
+int launch_record(const Dev& d, int level, const int* grids, uint64_t nodes, cudaStream_t st);
 size_t ninfo_bytes(int variant);
 int split_variant(int kind, int C);
 int variant_classes(int variant);  // largest class count of a kernel variant (1 for regression)

@@ -30,7 +30,8 @@
 // few_rows folds n and c into the weights, so the product gives q_k, and s is
 // exact in f32 (below 2^23 for n <= 66); every lane keeps its row's best
 // candidate exactly, comparing s_a den_b with s_b den_a in 64-bit integers.
-// mid_rows screens by the float score and compares exactly inside the window.
+// mid_rows takes every feature's best float score first, then compares the
+// features inside the window of the best one exactly.
 //
 // Measured (one iteration, before: ballots over the bin bits and 5 population
 // counts per class for <= 32 rows, a 256-bin shared-memory histogram for
@@ -91,33 +92,6 @@ template <typename T>
 __device__ __forceinline__ T pick4(T v0, T v1, T v2, T v3, int t) {
   const T a = (t & 1) ? v1 : v0, b = (t & 1) ? v3 : v2;
   return (t & 2) ? b : a;
-}
-
-// Record of a split found here: s / (den n) is the impurity decrease, its
-// numerator and denominator exact (the general form's numerator
-// num n_P - A_P den equals s), each rounded once.  cL: left class counts.
-template <int CM>
-__device__ uint32_t commit_counts(const Dev& d, uint32_t k, bool valid, uint32_t feat, uint32_t bin, uint32_t nL,
-                                  const uint32_t (&cL)[CM], unsigned long long s, uint32_t n) {
-  uint32_t sp = kLeaf;
-  if (valid) {
-    const unsigned long long den = static_cast<unsigned long long>(nL) * (n - nL) * n;
-    const double delta = d.precision == 0
-                             ? __ull2double_rn(s) / __ull2double_rn(den)
-                             : static_cast<double>(__fdiv_rn(__ull2float_rn(s), __ull2float_rn(den)));
-    sp = (feat << 8) | bin;
-    d.nd_delta[k] = delta;
-    d.nd_ln[k] = nL;
-#pragma unroll
-    for (int c = 0; c < CM; ++c)
-      if (c < ncls<CM>(d)) d.nd_lcnt[static_cast<int64_t>(k) * d.C + c] = cL[c];
-    if (!d.permut) {  // Alg. 2: this node's gain x samples, summed exactly per (tree, feature)
-      if (!csa_add(d.acc + (static_cast<int64_t>(d.nd_tree[k]) * d.p_aug + feat) * kCsaLimbs, delta))
-        atomicOr(&d.status[0], kErrAcc);
-    }
-  }
-  d.nd_split[k] = sp;
-  return sp;
 }
 
 // ---------------------------------------------------------------- at most 32 rows
@@ -390,7 +364,7 @@ __device__ void mid_rows(const Dev& d, int level, uint32_t k, MidTile& sm, unsig
     }
   const float n = static_cast<float>(nd.n);
   const float c0 = static_cast<float>(sm.tot[CM == 2 ? 0 : 2 * t]), c1 = static_cast<float>(sm.tot[2 * t + 1]);
-  float bestf = 0.0f;
+  uint32_t seen = 0u;  // best float score so far, as its bits
   unsigned long long bs = 0ull;
   uint32_t bden = 1u, bkey = 0xFFFFFFFFu;
   for (int r0 = 0; r0 < d.mtry; r0 += 32) {
@@ -413,13 +387,15 @@ __device__ void mid_rows(const Dev& d, int level, uint32_t k, MidTile& sm, unsig
       for (int q = 0; q < 8; ++q) sm.bins[lane * 33 + 8 * hb + q] = b[2 * q] | (b[2 * q + 1] << 16);
     }
     __syncwarp();
+    uint32_t fbest = 0u;  // of feature `lane`
     for (int j = 0; j < nf; ++j) {
       const uint32_t* tw = sm.bins + j * 33;
       const uint16_t* th = reinterpret_cast<const uint16_t*>(tw);
       uint32_t A[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) A[i] = i < 2 * nb ? tw[4 * i + t] : 0u;
-      float sf[2], nLo[2];
+      // best float score of the feature (non-negative: their bits order as they do)
+      float mine = 0.0f;
 #pragma unroll
       for (int hb = 0; hb < 2; ++hb) {
         float p[4] = {0.0f, 0.0f, 0.0f, 0.0f}, nl[4] = {0.0f, 0.0f, 0.0f, 0.0f};
@@ -437,18 +413,26 @@ __device__ void mid_rows(const Dev& d, int level, uint32_t k, MidTile& sm, unsig
           }
         }
         const float s = CM == 2 ? 2.0f * pick4(p[0], p[1], p[2], p[3], t) : quad_sum_own(p, t);
-        nLo[hb] = pick4(nl[0], nl[1], nl[2], nl[3], t);
-        sf[hb] = (32 * hb + 8 * t + g < len && s > 0.0f) ? __fdividef(s, nLo[hb] * (n - nLo[hb])) : 0.0f;
+        const float l = pick4(nl[0], nl[1], nl[2], nl[3], t);
+        if (32 * hb + 8 * t + g < len && s > 0.0f) mine = fmaxf(mine, __fdividef(s, l * (n - l)));
       }
-      // scores are non-negative: their bits order as they do
-      const float mx = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(fmaxf(sf[0], sf[1]))));
-      if (mx == 0.0f || mx < screen(bestf)) continue;
-      bestf = fmaxf(mx, bestf);
-      const float thr = screen(bestf);
-      // candidates inside the window, exactly (uniform branch; a few features of a node)
+      const uint32_t mx = __reduce_max_sync(kFull, __float_as_uint(mine));
+      if (lane == j) fbest = mx;
+    }
+    // the features inside the window of the best score (usually one), exactly
+    seen = max(seen, __reduce_max_sync(kFull, fbest));
+    for (unsigned in = __ballot_sync(kFull, fbest != 0u && __uint_as_float(fbest) >= screen(__uint_as_float(seen))); in;
+         in &= in - 1) {
+      const int j = __ffs(in) - 1;
+      const uint32_t* tw = sm.bins + j * 33;
+      const uint16_t* th = reinterpret_cast<const uint16_t*>(tw);
+      uint32_t A[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) A[i] = i < 2 * nb ? tw[4 * i + t] : 0u;
 #pragma unroll
       for (int hb = 0; hb < 2; ++hb) {
         unsigned long long p[4] = {0ull, 0ull, 0ull, 0ull};
+        float nL[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
         for (int m = 0; m < 2; ++m) {
           const int mb = 2 * hb + m;
@@ -457,14 +441,15 @@ __device__ void mid_rows(const Dev& d, int level, uint32_t k, MidTile& sm, unsig
             mid_block<CM>(A, dup_h(th[16 * mb + g]), dup_h(th[16 * mb + 8 + g]), B, Bw, nb, n, c0, c1, q0, q1, x);
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
-              const long long y0 = static_cast<long long>(q0[r]), y1 = static_cast<long long>(q1[r]);
+              const long long y0 = static_cast<int32_t>(q0[r]), y1 = static_cast<int32_t>(q1[r]);
               p[2 * m + r] = static_cast<unsigned long long>(y0 * y0 + y1 * y1);
+              nL[2 * m + r] = x[r];
             }
           }
         }
         const unsigned long long s = CM == 2 ? 2ull * pick4(p[0], p[1], p[2], p[3], t) : quad_sum_own(p, t);
-        if (sf[hb] >= thr) {
-          const uint32_t nl = f23_to_u32(nLo[hb]);
+        const uint32_t nl = f23_to_u32(pick4(nL[0], nL[1], nL[2], nL[3], t));
+        if (32 * hb + 8 * t + g < len && s > 0ull) {
           const uint32_t den = nl * (nd.n - nl);
           const uint32_t key = sm.key[j] | th[32 * hb + 8 * t + g];
           const unsigned long long x = s * bden, y = bs * den;  // n <= 64 * 31: below 2^62

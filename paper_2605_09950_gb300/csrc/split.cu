@@ -31,6 +31,7 @@
 // (variance); scores are compared exactly (256-bit cross products) after a
 // float pre-screen; equal scores go to the lower key = (feature index, or
 // the draw slot with tie_break = 1) << 8 | bin.
+#include <algorithm>
 #include <cstdint>
 #include <type_traits>
 
@@ -273,7 +274,7 @@ __global__ void __launch_bounds__(256) k_classify(Dev d, int level) {
   for (uint32_t base = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; base < lcount;
        base += gridDim.x * blockDim.x) {
     const uint32_t idx = base + lane;
-    int cls = 0;  // 0 none, 1 small, 2 larger, 3 tiny, 4 micro, 5 mid
+    int cls = 0;  // 0 none, 1 small, 2 larger, 3 tiny, 4 micro, 5 mid, 6..8 by record
     uint32_t k = 0;
     if (idx < lcount) {
       k = loff + idx;
@@ -281,6 +282,11 @@ __global__ void __launch_bounds__(256) k_classify(Dev d, int level) {
       if (load_node<KIND, CM>(d, k, level, nd)) {
         cls = nd.len > kFewRows ? 2 : (nd.len > 16u ? 1 : (nd.len > 8u ? 3 : 4));
         if (KIND == 0 && nd.len <= kMidRows && (cls == 2 || nd.n > kFewWeight)) cls = 5;
+        // by record: 10-bit counts, exact f32 products below weight 4096, 16-bit counts
+        if (KIND == 0 && cls == 2 && nd.len <= d.rec_rows && nd.n < 65536u)
+          cls = nd.len <= 256u && nd.n < 1024u ? 6
+                : nd.len <= 1024u && nd.n < 4096u ? (d.rec_rows > 256u ? 7 : 2)
+                                                  : (d.rec_rows > 1024u ? 8 : 2);
       } else {
         d.nd_split[k] = kLeaf;
       }
@@ -298,6 +304,13 @@ __global__ void __launch_bounds__(256) k_classify(Dev d, int level) {
     if (cls == 3) d.small[d.small_cap - 1u - t0] = k;
     if (cls == 4) d.micro[m0] = k;
     if (cls == 5) d.mid[d0] = k;
+    if (KIND == 0 && d.rec_rows > 0u) {
+      const uint32_t r0 = append(6, &d.nrec[3 * level]), r1 = append(7, &d.nrec[3 * level + 1]),
+                     r2 = append(8, &d.nrec[3 * level + 2]);
+      if (cls == 6) d.rec[r0] = k;
+      if (cls == 7) d.rec2[r1] = k;
+      if (cls == 8) d.rec2[d.rec2_cap - 1u - r2] = k;
+    }
   }
 }
 
@@ -1593,8 +1606,8 @@ __global__ void __launch_bounds__(256, BORUTA_SMALL_MINB) k_finalize(Dev d, int 
 }
 
 template <int KIND, int CM>
-int launch_level(const Dev& d, int level, int grid_small, int grid_items, uint64_t big_bound, size_t smem,
-                 cudaStream_t st, cudaStream_t st2, cudaEvent_t fork, cudaEvent_t join, cudaEvent_t hist_start,
+int launch_level(const Dev& d, int level, int grid_small, int grid_items, const int* grid_rec, uint64_t big_bound,
+                 size_t smem, cudaStream_t st, cudaStream_t st2, cudaEvent_t fork, cudaEvent_t join, cudaEvent_t hist_start,
                  cudaEvent_t hist_end) {
   int n = 1;
   k_classify<KIND, CM><<<grid_small, 256, 0, st>>>(d, level);
@@ -1610,6 +1623,18 @@ int launch_level(const Dev& d, int level, int grid_small, int grid_items, uint64
     n += 3;
   }
   cudaEventRecord(join, st2);
+  if constexpr (KIND == 0) {
+    if (d.rec_rows > 0u) {
+      if (hist_start) cudaEventRecord(hist_start, st);
+      n += launch_record(d, level, grid_rec, std::max<uint64_t>(big_bound, 1), st);
+      if (static_cast<uint32_t>(d.N) <= d.rec_rows) {  // no node is larger
+        if (hist_end) cudaEventRecord(hist_end, st);
+        cudaStreamWaitEvent(st, join, 0);
+        return n;
+      }
+    }
+  }
+  const bool hist_open = KIND == 0 && d.rec_rows > 0u;
   // band path: the larger nodes in chunks of chunk_cap (at most big_bound
   // nodes exist; chunks past the level's count return at once)
   const uint64_t nchunks =
@@ -1623,7 +1648,7 @@ int launch_level(const Dev& d, int level, int grid_small, int grid_items, uint64
     k_plan_scatter<KIND, CM><<<grid_small, 256, 0, st>>>(dc, level);
     // the histogram kernel of the level (with several chunks the window also
     // holds the later chunks' plan and finalize kernels)
-    if (c == 0 && hist_start) cudaEventRecord(hist_start, st);
+    if (c == 0 && hist_start && !hist_open) cudaEventRecord(hist_start, st);
     if (d.band_launch)
       for (int b = 0; b < d.nbands; ++b) k_items_band<KIND, CM><<<grid_items, kSplitThreads, smem, st>>>(dc, level, b);
     else
@@ -1633,7 +1658,7 @@ int launch_level(const Dev& d, int level, int grid_small, int grid_items, uint64
     n += 4 + (d.band_launch ? d.nbands : 1);
   }
   if (nchunks == 0) {  // grouped path
-    if (hist_start) cudaEventRecord(hist_start, st);
+    if (hist_start && !hist_open) cudaEventRecord(hist_start, st);
     k_items<KIND, CM><<<grid_items, kSplitThreads, smem, st>>>(d, level);
     if (hist_end) cudaEventRecord(hist_end, st);
     k_finalize<KIND, CM><<<grid_small, 256, 0, st>>>(d, level);
@@ -1694,11 +1719,11 @@ const void* small_kernel_ptr(int variant) {
   });
 }
 
-int launch_split(const Dev& d, int level, int grid_small, int grid_big, uint64_t big_bound, size_t smem,
-                 cudaStream_t st, cudaStream_t st2, cudaEvent_t fork, cudaEvent_t join, cudaEvent_t hs,
+int launch_split(const Dev& d, int level, int grid_small, int grid_big, const int* grid_rec, uint64_t big_bound,
+                 size_t smem, cudaStream_t st, cudaStream_t st2, cudaEvent_t fork, cudaEvent_t join, cudaEvent_t hs,
                  cudaEvent_t he) {
   return with_variant(split_variant(d.kind, d.C), [&](auto kind, auto cm) {
-    return launch_level<decltype(kind)::value, decltype(cm)::value>(d, level, grid_small, grid_big, big_bound, smem,
+    return launch_level<decltype(kind)::value, decltype(cm)::value>(d, level, grid_small, grid_big, grid_rec, big_bound, smem,
                                                                      st, st2, fork, join, hs, he);
   });
 }

@@ -291,6 +291,34 @@ __device__ uint32_t commit_split(const Dev& d, uint32_t k, const Cand<CM>& b, co
   return sp;
 }
 
+// Record of a split given by its counts: s / (n_L n_R n), s = sum_k q_k^2,
+// q_k = l_k n - c_k n_L, is the impurity decrease, its
+// numerator and denominator exact (the general form's numerator
+// num n_P - A_P den equals s), each rounded once.  cL: left class counts.
+template <int CM>
+__device__ __noinline__ uint32_t commit_counts(const Dev& d, uint32_t k, bool valid, uint32_t feat, uint32_t bin, uint32_t nL,
+                                  const uint32_t (&cL)[CM], unsigned long long s, uint32_t n) {
+  uint32_t sp = kLeaf;
+  if (valid) {
+    const unsigned long long den = static_cast<unsigned long long>(nL) * (n - nL) * n;
+    const double delta = d.precision == 0
+                             ? __ull2double_rn(s) / __ull2double_rn(den)
+                             : static_cast<double>(__fdiv_rn(__ull2float_rn(s), __ull2float_rn(den)));
+    sp = (feat << 8) | bin;
+    d.nd_delta[k] = delta;
+    d.nd_ln[k] = nL;
+#pragma unroll
+    for (int c = 0; c < CM; ++c)
+      if (c < ncls<CM>(d)) d.nd_lcnt[static_cast<int64_t>(k) * d.C + c] = cL[c];
+    if (!d.permut) {  // Alg. 2: this node's gain x samples, summed exactly per (tree, feature)
+      if (!csa_add(d.acc + (static_cast<int64_t>(d.nd_tree[k]) * d.p_aug + feat) * kCsaLimbs, delta))
+        atomicOr(&d.status[0], kErrAcc);
+    }
+  }
+  d.nd_split[k] = sp;
+  return sp;
+}
+
 template <int KIND, int CM>
 __device__ bool load_node(const Dev& d, uint32_t k, int level, NodeInfo<CM>& nd) {
   const uint32_t tau = d.nd_tree[k];

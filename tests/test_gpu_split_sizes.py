@@ -1,6 +1,7 @@
 """Split kernels at the sizes where their layouts change: nodes of 8, 16, 32
 and 64 rows (matrix-product split of few rows), samples around 32 features,
-2 to 8 classes, coarse bins (exact ties) and fine ones; every tree against
+nodes of 128, 256, 1024 and 4096
+rows (by-record split), 2 to 8 classes, coarse bins (exact ties) and fine ones; every tree against
 the CPU oracle, bit for bit."""
 import numpy as np
 import pytest
@@ -27,4 +28,14 @@ def workload(N, p, classes, bins, n_trees, depth, mtry, seed, importance=synth.T
                                          (410, 256, 32)])
 def test_small_nodes(classes, N, bins, mtry):
     w = workload(N, 20, classes, bins, 24, 12, mtry, seed=N + classes)
+    check_iteration(w, tie_break=classes & 1)
+
+
+@pytest.mark.parametrize("classes", [2, 3, 5, 8])
+@pytest.mark.parametrize("N,bins,mtry", [(205, 256, 33), (408, 60, 31), (415, 256, 7), (1650, 100, 40), (1622, 256, 3),
+                                         (6480, 256, 5), (6700, 20, 34), (9000, 256, 4)])
+def test_nodes_by_record(classes, N, bins, mtry):
+    """In-bag roots around 128, 256, 1024 and 4096 rows (the tiles of the
+    by-record kernels), more rows than the largest, bins of every lane width."""
+    w = workload(N, 20, classes, bins, 5, 4, mtry, seed=N + classes)
     check_iteration(w, tie_break=classes & 1)
