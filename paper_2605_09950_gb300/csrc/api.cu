@@ -97,7 +97,7 @@ struct boruta_session {
   // launch geometry
   int sms = 0, split_grid = 0, small_grid = 0, tree_grid = 0, permut_grid = 0, walk_grid = 0;
   size_t split_smem = 0;
-  int rec_grid[3] = {0, 0, 0};  // blocks of the three by-record kernels that the GPU holds at once
+  int rec_grid[3] = {0, 0, 0};  // blocks of record.cu's or threebin.cu's kernels that the GPU holds at once
   // second stream for the small-node kernel, and its fork/join events
   cudaStream_t st2 = nullptr;
   cudaEvent_t fork = nullptr, join = nullptr;
@@ -439,7 +439,10 @@ static int session_init(boruta_session* s, const uint8_t* X, int64_t ld, const v
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kptr[1], kSplitThreads, s->split_smem));
   if (per_sm < 1) return fail(BORUTA_EINVAL, "split kernel does not fit on an SM");
   s->split_grid = per_sm * s->sms;
-  if (!reg) CK(static_cast<cudaError_t>(setup_record(variant, s->sms, s->rec_grid)));
+  if (!reg)
+    CK(static_cast<cudaError_t>(setup_record(variant, s->sms, s->rec_grid)));
+  else if (d.B <= 3)
+    CK(static_cast<cudaError_t>(setup_three_bins(static_cast<int>(p_aug_max), s->sms, s->rec_grid)));
   // warp-per-node kernels: as many blocks as the GPU holds at once (they
   // loop over their nodes), so no partial last wave
   int small_per_sm = 0;
@@ -524,6 +527,9 @@ static int enqueue_iteration(boruta_session* s, int t, cudaStream_t st) {
   d.mtry = static_cast<int32_t>(std::max<int64_t>(m, 1));
   d.ldP = static_cast<int32_t>((p_aug + 15) / 16 * 16);
   d.rec_rows = record_rows(s, d);
+  // threebin.cu reads whole records: at most 8 times the sampled columns
+  d.three_bins = d.kind == 1 && d.B <= 3 && s->split_path == 0 && s->rec_grid[0] > 0 && s->rec_grid[1] > 0 &&
+                 8ll * d.mtry >= p_aug;
   // feature bands: ~kBandBytes of columns each, at most kMaxBands; the packed
   // item holds a 14-bit slot and a 22-bit feature
   d.band_w = 0;
@@ -620,7 +626,7 @@ static int enqueue_iteration(boruta_session* s, int t, cudaStream_t st) {
     }
     s->used_bw[level] = dl.band_w;
     s->used_bl[level] = dl.band_launch;
-    nk += launch_split(dl, level, std::max(gs, 1), gi, s->rec_grid, big, s->split_smem, st, s->st2, s->fork, s->join,
+    nk += launch_split(dl, level, std::max(gs, 1), gi, s->rec_grid, nodes, big, s->split_smem, st, s->st2, s->fork, s->join,
                        timed ? s->hev[2 * level] : nullptr, timed ? s->hev[2 * level + 1] : nullptr);
     CK_LAUNCH("split kernels");
     if (timed) CK(cudaEventRecord(s->ev[2 * level + 1], st));

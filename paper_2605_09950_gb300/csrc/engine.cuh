@@ -64,6 +64,8 @@ struct Dev {
   uint32_t* nrec;                // [D + 2][3] per level: numbers of the three
   uint32_t rec2_cap;
   uint32_t rec_rows;             // largest node split by record (0: none)
+  int32_t three_bins;            // 1: regression nodes below kThreeRows rows go to threebin.cu, those of at
+                                 //   most 8 rows listed in `micro`, the others in `small`
   uint32_t small_cap;            // entries of `small`
   void* ninfo;                   // [big_cap] node totals of `big`, by rank
   void* cand;                    // [big_cap * kItemsPerNode] best candidate per grouped item
@@ -104,6 +106,7 @@ struct Dev {
 // half precision (at most 2048).
 constexpr uint32_t kFewRows = 32, kFewWeight = 66, kMidRows = 64;
 constexpr uint32_t kRecordRows = 4096;  // largest node of record.cu
+constexpr uint32_t kThreeRows = 16384;  // nodes of threebin.cu have fewer rows (its f32 limb sums)
 constexpr int kScanBlocks = 512;
 constexpr int kSplitThreads = 256;
 constexpr int kItemsPerNode = 16;  // work items (groups of draw slots) per larger node
@@ -129,8 +132,8 @@ int launch_bootstrap(const Dev& d, int grid, cudaStream_t st);
 // small-node kernel then runs on `st2` while the larger-node kernels run on
 // `st` (fork/join through the two events).
 // hist_start/hist_end are recorded on `st` around the histogram kernel.
-int launch_split(const Dev& d, int level, int grid_small, int grid_big, const int* grid_rec, uint64_t big_bound,
-                  size_t smem, cudaStream_t st,
+int launch_split(const Dev& d, int level, int grid_small, int grid_big, const int* grid_rec, uint64_t nodes,
+                  uint64_t big_bound, size_t smem, cudaStream_t st,
                   cudaStream_t st2, cudaEvent_t fork, cudaEvent_t join, cudaEvent_t hist_start,
                   cudaEvent_t hist_end);
 // small.cu: the level's classification nodes of few rows, on `st`
@@ -139,6 +142,10 @@ int launch_few_rows(const Dev& d, int level, int grid, cudaStream_t st);
 // level's larger classification nodes of at most rec_rows rows, on `st`
 int setup_record(int variant, int sms, int* grids);
 int launch_record(const Dev& d, int level, const int* grids, uint64_t nodes, cudaStream_t st);
+// threebin.cu: grid sizes for at most p_aug columns; the level's regression
+// nodes below kThreeRows rows, the smallest on `st2`
+int setup_three_bins(int p_aug, int sms, int* grids);
+int launch_three_bins(const Dev& d, int level, const int* grids, uint64_t nodes, cudaStream_t st, cudaStream_t st2);
 size_t ninfo_bytes(int variant);
 int split_variant(int kind, int C);
 int variant_classes(int variant);  // largest class count of a kernel variant (1 for regression)

@@ -281,6 +281,7 @@ __global__ void __launch_bounds__(256) k_classify(Dev d, int level) {
       NodeInfo<CM> nd;
       if (load_node<KIND, CM>(d, k, level, nd)) {
         cls = nd.len > kFewRows ? 2 : (nd.len > 16u ? 1 : (nd.len > 8u ? 3 : 4));
+        if (KIND == 1 && d.three_bins) cls = nd.len >= kThreeRows ? 2 : (nd.len > 8u ? 1 : 4);
         if (KIND == 0 && nd.len <= kMidRows && (cls == 2 || nd.n > kFewWeight)) cls = 5;
         // by record: 10-bit counts, exact f32 products below weight 4096, 16-bit counts
         if (KIND == 0 && cls == 2 && nd.len <= d.rec_rows && nd.n < 65536u)
@@ -1606,8 +1607,8 @@ __global__ void __launch_bounds__(256, BORUTA_SMALL_MINB) k_finalize(Dev d, int 
 }
 
 template <int KIND, int CM>
-int launch_level(const Dev& d, int level, int grid_small, int grid_items, const int* grid_rec, uint64_t big_bound,
-                 size_t smem, cudaStream_t st, cudaStream_t st2, cudaEvent_t fork, cudaEvent_t join, cudaEvent_t hist_start,
+int launch_level(const Dev& d, int level, int grid_small, int grid_items, const int* grid_rec, uint64_t nodes,
+                 uint64_t big_bound, size_t smem, cudaStream_t st, cudaStream_t st2, cudaEvent_t fork, cudaEvent_t join, cudaEvent_t hist_start,
                  cudaEvent_t hist_end) {
   int n = 1;
   k_classify<KIND, CM><<<grid_small, 256, 0, st>>>(d, level);
@@ -1616,6 +1617,9 @@ int launch_level(const Dev& d, int level, int grid_small, int grid_items, const 
   cudaStreamWaitEvent(st2, fork, 0);
   if constexpr (KIND == 0) {
     n += launch_few_rows(d, level, grid_small, st2);
+  } else if (d.three_bins) {
+    if (hist_start) cudaEventRecord(hist_start, st);
+    n += launch_three_bins(d, level, grid_rec, nodes, st, st2);
   } else {
     k_split_small<KIND, CM, 8><<<grid_small, 256, 0, st2>>>(d, level);
     k_split_small<KIND, CM, 16><<<grid_small, 256, 0, st2>>>(d, level);
@@ -1634,7 +1638,12 @@ int launch_level(const Dev& d, int level, int grid_small, int grid_items, const 
       }
     }
   }
-  const bool hist_open = KIND == 0 && d.rec_rows > 0u;
+  if (KIND == 1 && d.three_bins && static_cast<uint32_t>(d.N) < kThreeRows) {  // no node is larger
+    if (hist_end) cudaEventRecord(hist_end, st);
+    cudaStreamWaitEvent(st, join, 0);
+    return n;
+  }
+  const bool hist_open = KIND == 0 ? d.rec_rows > 0u : d.three_bins != 0;
   // band path: the larger nodes in chunks of chunk_cap (at most big_bound
   // nodes exist; chunks past the level's count return at once)
   const uint64_t nchunks =
@@ -1719,11 +1728,11 @@ const void* small_kernel_ptr(int variant) {
   });
 }
 
-int launch_split(const Dev& d, int level, int grid_small, int grid_big, const int* grid_rec, uint64_t big_bound,
-                 size_t smem, cudaStream_t st, cudaStream_t st2, cudaEvent_t fork, cudaEvent_t join, cudaEvent_t hs,
+int launch_split(const Dev& d, int level, int grid_small, int grid_big, const int* grid_rec, uint64_t nodes,
+                 uint64_t big_bound, size_t smem, cudaStream_t st, cudaStream_t st2, cudaEvent_t fork, cudaEvent_t join, cudaEvent_t hs,
                  cudaEvent_t he) {
   return with_variant(split_variant(d.kind, d.C), [&](auto kind, auto cm) {
-    return launch_level<decltype(kind)::value, decltype(cm)::value>(d, level, grid_small, grid_big, grid_rec, big_bound, smem,
+    return launch_level<decltype(kind)::value, decltype(cm)::value>(d, level, grid_small, grid_big, grid_rec, nodes, big_bound, smem,
                                                                      st, st2, fork, join, hs, he);
   });
 }

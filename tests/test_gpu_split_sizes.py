@@ -39,3 +39,22 @@ def test_nodes_by_record(classes, N, bins, mtry):
     by-record kernels), more rows than the largest, bins of every lane width."""
     w = workload(N, 20, classes, bins, 5, 4, mtry, seed=N + classes)
     check_iteration(w, tie_break=classes & 1)
+
+
+@pytest.mark.parametrize("tie_break", [0, 1])
+@pytest.mark.parametrize("N,p,bins,discrete", [(13, 3, 3, 0), (30, 70, 2, 0), (900, 40, 3, 0), (900, 200, 3, 1),
+                                               (2500, 130, 3, 0), (27_000, 5, 3, 0)])
+def test_three_bin_regression(N, p, bins, discrete, tie_break):
+    """Genotype columns: nodes of at most 8 rows, of one and several staged
+    chunks and above the matrix-product kernel's largest (16384 rows); column
+    counts around 128; few distinct targets (exact ties of unlike subsets)."""
+    rng = np.random.default_rng(N + p)
+    X = np.zeros((p, synth.pad16(N)), np.uint8)
+    X[:, :N] = rng.integers(0, bins, size=(p, N))
+    y = X[0, :N].astype(np.int64) * 3 - X[p // 2, :N] + (rng.integers(-2, 3, N) if discrete else 0)
+    y = y * 2**20 + (0 if discrete else rng.integers(-2**23, 2**23, N))
+    if N == 13:
+        y = y * 2**33 - 2**55  # large targets: every limb in use
+    w = synth.Workload("t", X, y.astype(np.int64), N, p, synth.REGRESSION | synth.TREEIMP, 1, bins, 6 if N < 5000 else 2,
+                       9 if N < 5000 else 2, 2, seed=N, mtry=0)
+    check_iteration(w, tie_break=tie_break)
