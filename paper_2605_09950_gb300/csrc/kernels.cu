@@ -136,10 +136,15 @@ int launch_gather_live(const Dev& d, cudaStream_t st) {
 }
 
 // Xaug[p_live + c][i] = X[sigma_c(i)][live[c mod p_live]]; 16 rows per thread, one
-// 16-byte store.  The source column is read through L2 (random gather).
+// 16-byte store.  The source column is read through L2 (random gather).  A
+// row's cycle walk leaves the domain [0, 4^h) of the network 4^h / N times on
+// average; a thread goes on to its next row as soon as its walk ends, so the
+// warp waits for the longest sum of 16 walks, not 16 times for the longest
+// walk (N = 1e5, 1000 columns: 3.0 -> 1.35 ms).
 __global__ void k_shadow(Dev d) {
   const int c = blockIdx.y;
   __shared__ Perm sp;
+  __shared__ uint32_t at[16][256];  // a thread's 16 source rows
   if (threadIdx.x == 0)
     perm_init(sp, static_cast<uint32_t>(d.N), d.seed, 0u, unit_word(d.t, c),
               purpose_word(kPurposeShadow, d.job));
@@ -149,12 +154,20 @@ __global__ void k_shadow(Dev d) {
   uint8_t* dst = d.Xaug + static_cast<int64_t>(d.p_live + c) * d.ldN;
   for (int base = (blockIdx.x * blockDim.x + threadIdx.x) * 16; base < d.N;
        base += gridDim.x * blockDim.x * 16) {
+    const int rows = min(16, d.N - base);
+    uint32_t x = static_cast<uint32_t>(base);
+    for (int k = 0; k < rows;) {
+      if (P.n > 1u) x = feistel8(P, x);
+      if (x < P.n) {
+        at[k][threadIdx.x] = x;
+        ++k;
+        x = static_cast<uint32_t>(base + k);
+      }
+    }
     uint32_t v[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      const int i = base + k;
-      if (i < d.N) v[k >> 2] |= static_cast<uint32_t>(src[perm_apply(P, i)]) << (8 * (k & 3));
-    }
+    for (int k = 0; k < 16; ++k)
+      if (k < rows) v[k >> 2] |= static_cast<uint32_t>(src[at[k][threadIdx.x]]) << (8 * (k & 3));
     *reinterpret_cast<uint4*>(dst + base) = make_uint4(v[0], v[1], v[2], v[3]);
   }
 }
