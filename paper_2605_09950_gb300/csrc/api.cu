@@ -344,6 +344,7 @@ static int session_init(boruta_session* s, const uint8_t* X, int64_t ld, const v
   d.B = std::max(2, std::min(n_bins, static_cast<int>(s->status_h[3]) + 1));
   if (reg) {
     d.C = 1;
+    d.wide_y = maxy >= (1ull << 33);  // 255 maxy: 41 bits and a sign (regress.cu)
     if (maxy && static_cast<double>(maxy) * static_cast<double>(N) >= 4611686018427387904.0)
       return fail(BORUTA_EOVERFLOW, "N * max|y| must stay below 2^62");
   } else {
@@ -368,11 +369,11 @@ static int session_init(boruta_session* s, const uint8_t* X, int64_t ld, const v
     const size_t mid_cap = static_cast<size_t>(N) / (kFewRows + 1) + static_cast<size_t>(N) / (kFewWeight + 1) + 2;
     if ((rc = s->alloc(&d.mid, static_cast<size_t>(n_trees) * mid_cap))) return rc;
     if ((rc = s->alloc(&d.nmid, max_depth + 2))) return rc;
-    if ((rc = s->alloc(&d.rec, static_cast<size_t>(n_trees) * (static_cast<size_t>(N) / (kMidRows + 1) + 1)))) return rc;
-    d.rec2_cap = static_cast<uint32_t>(n_trees) * (static_cast<uint32_t>(N) / 257u + 2u);
-    if ((rc = s->alloc(&d.rec2, d.rec2_cap))) return rc;
-    if ((rc = s->alloc(&d.nrec, 3 * (max_depth + 2)))) return rc;
   }
+  if ((rc = s->alloc(&d.rec, static_cast<size_t>(n_trees) * (static_cast<size_t>(N) / (big_rows + 1) + 1)))) return rc;
+  d.rec2_cap = static_cast<uint32_t>(n_trees) * (static_cast<uint32_t>(N) / 257u + 2u);
+  if ((rc = s->alloc(&d.rec2, d.rec2_cap))) return rc;
+  if ((rc = s->alloc(&d.nrec, 3 * (max_depth + 2)))) return rc;
   if ((rc = s->alloc(&d.big, big_cap))) return rc;
   uint8_t* ninfo = nullptr;
   if ((rc = s->alloc(&ninfo, big_cap * ninfo_bytes(split_variant(d.kind, d.C))))) return rc;
@@ -443,6 +444,8 @@ static int session_init(boruta_session* s, const uint8_t* X, int64_t ld, const v
     CK(static_cast<cudaError_t>(setup_record(variant, s->sms, s->rec_grid)));
   else if (d.B <= 3)
     CK(static_cast<cudaError_t>(setup_three_bins(static_cast<int>(p_aug_max), s->sms, s->rec_grid)));
+  else
+    CK(static_cast<cudaError_t>(setup_regress(s->sms, s->rec_grid)));
   // warp-per-node kernels: as many blocks as the GPU holds at once (they
   // loop over their nodes), so no partial last wave
   int small_per_sm = 0;
@@ -530,6 +533,10 @@ static int enqueue_iteration(boruta_session* s, int t, cudaStream_t st) {
   // threebin.cu reads whole records: at most 8 times the sampled columns
   d.three_bins = d.kind == 1 && d.B <= 3 && s->split_path == 0 && s->rec_grid[0] > 0 && s->rec_grid[1] > 0 &&
                  8ll * d.mtry >= p_aug;
+  // regress.cu: columns of more than 4 bins (fewer are counted in registers by
+  // the column path), lists of 16-bit columns
+  if (d.kind == 1 && d.B > 4 && s->split_path == 0 && d.mtry <= kRegColumns && p_aug <= 65536)
+    d.rec_rows = std::min<uint32_t>(kRegRecordRows, static_cast<uint32_t>(d.N));
   // feature bands: ~kBandBytes of columns each, at most kMaxBands; the packed
   // item holds a 14-bit slot and a 22-bit feature
   d.band_w = 0;
@@ -586,7 +593,7 @@ static int enqueue_iteration(boruta_session* s, int t, cudaStream_t st) {
   CK(cudaMemsetAsync(d.ntiny, 0, (d.D + 2) * sizeof(uint32_t), st));
   CK(cudaMemsetAsync(d.nmicro, 0, (d.D + 2) * sizeof(uint32_t), st));
   if (d.nmid) CK(cudaMemsetAsync(d.nmid, 0, (d.D + 2) * sizeof(uint32_t), st));
-  if (d.nrec) CK(cudaMemsetAsync(d.nrec, 0, 3 * (d.D + 2) * sizeof(uint32_t), st));
+  CK(cudaMemsetAsync(d.nrec, 0, 3 * (d.D + 2) * sizeof(uint32_t), st));
   CK(cudaMemsetAsync(d.lvl_cnt, 0, (d.D + 2) * sizeof(uint32_t), st));
   CK(cudaMemsetAsync(d.counters, 0, 4 * sizeof(unsigned long long), st));
 

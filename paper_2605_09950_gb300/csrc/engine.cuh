@@ -59,11 +59,12 @@ struct Dev {
   uint32_t* mid;                 // [mid_cap] classification: nodes of 33..64 rows, and smaller ones
                                  //   whose weight exceeds kFewWeight
   uint32_t* nmid;                // [D + 2] per level: number of them
-  uint32_t* rec;                 // classification nodes split by record (record.cu): of 65..256 rows
+  uint32_t* rec;                 // nodes split by record: of 65..256 rows (record.cu), 33..256 (regress.cu)
   uint32_t* rec2;                // [rec2_cap] of 257..1024 rows (from its start), of up to 4096 (from its end)
   uint32_t* nrec;                // [D + 2][3] per level: numbers of the three
   uint32_t rec2_cap;
   uint32_t rec_rows;             // largest node split by record (0: none)
+  int32_t wide_y;                // regression: a row's weighted target may exceed 41 bits and its sign
   int32_t three_bins;            // 1: regression nodes below kThreeRows rows go to threebin.cu, those of at
                                  //   most 8 rows listed in `micro`, the others in `small`
   uint32_t small_cap;            // entries of `small`
@@ -107,6 +108,8 @@ struct Dev {
 constexpr uint32_t kFewRows = 32, kFewWeight = 66, kMidRows = 64;
 constexpr uint32_t kRecordRows = 4096;  // largest node of record.cu
 constexpr uint32_t kThreeRows = 16384;  // nodes of threebin.cu have fewer rows (its f32 limb sums)
+constexpr uint32_t kRegRecordRows = 1024;  // largest node of regress.cu (its 32-bit limb sums)
+constexpr int kRegColumns = 512;           // most sampled columns of regress.cu (its lists)
 constexpr int kScanBlocks = 512;
 constexpr int kSplitThreads = 256;
 constexpr int kItemsPerNode = 16;  // work items (groups of draw slots) per larger node
@@ -146,6 +149,10 @@ int launch_record(const Dev& d, int level, const int* grids, uint64_t nodes, cud
 // nodes below kThreeRows rows, the smallest on `st2`
 int setup_three_bins(int p_aug, int sms, int* grids);
 int launch_three_bins(const Dev& d, int level, const int* grids, uint64_t nodes, cudaStream_t st, cudaStream_t st2);
+// regress.cu: grid sizes; the level's regression nodes of at most rec_rows
+// rows (d.rec_rows > 0), those of at most 32 on `st2`
+int setup_regress(int sms, int* grids);
+int launch_regress(const Dev& d, int level, const int* grids, uint64_t nodes, cudaStream_t st, cudaStream_t st2);
 size_t ninfo_bytes(int variant);
 int split_variant(int kind, int C);
 int variant_classes(int variant);  // largest class count of a kernel variant (1 for regression)

@@ -125,36 +125,6 @@ struct RecordBest {
   uint32_t cum[Pack<CM, ROWS>::W];
 };
 
-// A lane's bpl (1, 2, 4 or 8) consecutive bins of a plane.
-__device__ __forceinline__ void ld_bins(const uint32_t* p, int bpl, uint32_t (&h)[8]) {
-#pragma unroll
-  for (int q = 0; q < 8; ++q) h[q] = 0u;
-  if (bpl >= 4) {
-    const uint4 a = reinterpret_cast<const uint4*>(p)[0];
-    h[0] = a.x, h[1] = a.y, h[2] = a.z, h[3] = a.w;
-    if (bpl == 8) {
-      const uint4 b = reinterpret_cast<const uint4*>(p)[1];
-      h[4] = b.x, h[5] = b.y, h[6] = b.z, h[7] = b.w;
-    }
-  } else if (bpl == 2) {
-    const uint2 a = *reinterpret_cast<const uint2*>(p);
-    h[0] = a.x, h[1] = a.y;
-  } else {
-    h[0] = *p;
-  }
-}
-
-__device__ __forceinline__ void st_bins(uint32_t* p, int bpl, const uint32_t (&h)[8]) {
-  if (bpl >= 4) {
-    reinterpret_cast<uint4*>(p)[0] = make_uint4(h[0], h[1], h[2], h[3]);
-    if (bpl == 8) reinterpret_cast<uint4*>(p)[1] = make_uint4(h[4], h[5], h[6], h[7]);
-  } else if (bpl == 2) {
-    *reinterpret_cast<uint2*>(p) = make_uint2(h[0], h[1]);
-  } else {
-    *p = h[0];
-  }
-}
-
 // A feature's histogram by one warp (zero on entry).
 template <int CM, int ROWS>
 __device__ __forceinline__ void record_count(const uint32_t* tile, const uint32_t* rw, uint32_t* hw, uint32_t len) {
@@ -198,8 +168,6 @@ __device__ __forceinline__ void record_zero(uint32_t* hw, int bpl) {
   for (int w = 0; w < Pack<CM, ROWS>::W; ++w) st_bins(hw + 256 * w + (threadIdx.x & 31) * bpl, bpl, zero);
   __syncwarp();
 }
-
-__device__ __forceinline__ int lane_bins(int B) { return B > 128 ? 8 : (B > 64 ? 4 : (B > 32 ? 2 : 1)); }
 
 // The exact best of a feature into the lanes' bests (the one or two features
 // of a node whose float best lies inside the window).
@@ -289,7 +257,6 @@ __device__ __forceinline__ void record_node(const Dev& d, int level, uint32_t k,
   constexpr int NW = Pk::W, CH = ROWS / (32 * WARPS), PITCH = ROWS / 4 + 1;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t* rows_in = d.rows[level & 1];
-  uint32_t* rows_out = d.rows[(level & 1) ^ 1];
   NodeInfo<CM> nd;
   load_node<0, CM>(d, k, level, nd);
   const uint32_t len = nd.len, chunks = (len + 31u) / 32u;
@@ -415,44 +382,13 @@ __device__ __forceinline__ void record_node(const Dev& d, int level, uint32_t k,
   __syncthreads();
   const uint32_t sp = sm.split;
   if (sp != kLeaf) {
-    // stable partition: left rows in order, then right rows in order
     const bool in_tile = d.mtry <= 32;
     const uint8_t* tb = reinterpret_cast<const uint8_t*>(sm.tile + sm.slot * PITCH);
-    unsigned bl[CH];
-#pragma unroll
-    for (int i = 0; i < CH; ++i) {
-      const uint32_t c = warp + WARPS * i, r = c * 32u + lane;
-      bl[i] = 0u;
-      if (c < chunks) {
-        uint32_t b = 256u;
-        if (r < len) b = in_tile ? tb[r] : row_bin(d, e[i] >> 8, sp >> 8);
-        bl[i] = __ballot_sync(kFull, b <= (sp & 255u));
-        if (lane == 0) sm.left[c] = __popc(bl[i]);
-      }
-    }
-    __syncthreads();
-    uint32_t total = 0u, before[CH];
-#pragma unroll
-    for (int i = 0; i < CH; ++i) before[i] = 0u;
-    for (uint32_t c0 = 0; c0 < chunks; c0 += 32u) {
-      const uint32_t v = c0 + lane < chunks ? sm.left[c0 + lane] : 0u;
-      const uint32_t x = total + warp_excl_scan_u32(v, lane);
-#pragma unroll
-      for (int i = 0; i < CH; ++i) {
-        const uint32_t c = warp + WARPS * i;
-        const uint32_t y = __shfl_sync(kFull, x, c & 31u);
-        if (c >= c0 && c < c0 + 32u) before[i] = y;
-      }
-      total = __shfl_sync(kFull, x + v, 31);
-    }
-#pragma unroll
-    for (int i = 0; i < CH; ++i) {
-      const uint32_t c = warp + WARPS * i, r = c * 32u + lane;
-      if (c < chunks && r < len) {
-        const uint32_t l = before[i] + __popc(bl[i] & lanemask_lt());
-        rows_out[nd.base + (((bl[i] >> lane) & 1u) ? l : total + (r - l))] = e[i];
-      }
-    }
+    const uint32_t total = block_partition<CH, WARPS>(
+        e, len, nd.base, d.rows[(level & 1) ^ 1], sm.left,
+        [&](int i, uint32_t r) {
+          return (in_tile ? static_cast<uint32_t>(tb[r]) : row_bin(d, e[i] >> 8, sp >> 8)) <= (sp & 255u);
+        });
     if (threadIdx.x == 0) d.nd_lrows[k] = total;
   }
   __syncthreads();  // the next node refills the block's shared memory

@@ -282,6 +282,7 @@ __global__ void __launch_bounds__(256) k_classify(Dev d, int level) {
       if (load_node<KIND, CM>(d, k, level, nd)) {
         cls = nd.len > kFewRows ? 2 : (nd.len > 16u ? 1 : (nd.len > 8u ? 3 : 4));
         if (KIND == 1 && d.three_bins) cls = nd.len >= kThreeRows ? 2 : (nd.len > 8u ? 1 : 4);
+        if (KIND == 1 && cls == 2 && nd.len <= d.rec_rows) cls = nd.len > 256u ? 7 : 6;
         if (KIND == 0 && nd.len <= kMidRows && (cls == 2 || nd.n > kFewWeight)) cls = 5;
         // by record: 10-bit counts, exact f32 products below weight 4096, 16-bit counts
         if (KIND == 0 && cls == 2 && nd.len <= d.rec_rows && nd.n < 65536u)
@@ -305,7 +306,7 @@ __global__ void __launch_bounds__(256) k_classify(Dev d, int level) {
     if (cls == 3) d.small[d.small_cap - 1u - t0] = k;
     if (cls == 4) d.micro[m0] = k;
     if (cls == 5) d.mid[d0] = k;
-    if (KIND == 0 && d.rec_rows > 0u) {
+    if (d.rec_rows > 0u) {
       const uint32_t r0 = append(6, &d.nrec[3 * level]), r1 = append(7, &d.nrec[3 * level + 1]),
                      r2 = append(8, &d.nrec[3 * level + 2]);
       if (cls == 6) d.rec[r0] = k;
@@ -1615,11 +1616,17 @@ int launch_level(const Dev& d, int level, int grid_small, int grid_items, const 
   // small nodes on st2, concurrently with the larger-node kernels on st
   cudaEventRecord(fork, st);
   cudaStreamWaitEvent(st2, fork, 0);
+  // rows of the largest node that the kernels of the other files take
+  const uint32_t taken = KIND == 1 && d.three_bins ? kThreeRows - 1u : d.rec_rows;
+  const bool hist_open = taken > 0u;
+  if (hist_open && hist_start) cudaEventRecord(hist_start, st);
   if constexpr (KIND == 0) {
     n += launch_few_rows(d, level, grid_small, st2);
+    if (d.rec_rows > 0u) n += launch_record(d, level, grid_rec, std::max<uint64_t>(big_bound, 1), st);
   } else if (d.three_bins) {
-    if (hist_start) cudaEventRecord(hist_start, st);
     n += launch_three_bins(d, level, grid_rec, nodes, st, st2);
+  } else if (d.rec_rows > 0u) {
+    n += launch_regress(d, level, grid_rec, nodes, st, st2);
   } else {
     k_split_small<KIND, CM, 8><<<grid_small, 256, 0, st2>>>(d, level);
     k_split_small<KIND, CM, 16><<<grid_small, 256, 0, st2>>>(d, level);
@@ -1627,23 +1634,11 @@ int launch_level(const Dev& d, int level, int grid_small, int grid_items, const 
     n += 3;
   }
   cudaEventRecord(join, st2);
-  if constexpr (KIND == 0) {
-    if (d.rec_rows > 0u) {
-      if (hist_start) cudaEventRecord(hist_start, st);
-      n += launch_record(d, level, grid_rec, std::max<uint64_t>(big_bound, 1), st);
-      if (static_cast<uint32_t>(d.N) <= d.rec_rows) {  // no node is larger
-        if (hist_end) cudaEventRecord(hist_end, st);
-        cudaStreamWaitEvent(st, join, 0);
-        return n;
-      }
-    }
-  }
-  if (KIND == 1 && d.three_bins && static_cast<uint32_t>(d.N) < kThreeRows) {  // no node is larger
+  if (static_cast<uint32_t>(d.N) <= taken) {  // no node is larger
     if (hist_end) cudaEventRecord(hist_end, st);
     cudaStreamWaitEvent(st, join, 0);
     return n;
   }
-  const bool hist_open = KIND == 0 ? d.rec_rows > 0u : d.three_bins != 0;
   // band path: the larger nodes in chunks of chunk_cap (at most big_bound
   // nodes exist; chunks past the level's count return at once)
   const uint64_t nchunks =

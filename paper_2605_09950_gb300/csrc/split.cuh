@@ -380,6 +380,84 @@ __device__ uint32_t warp_partition(const Dev& d, int64_t base, uint32_t len, uin
   return lbase;
 }
 
+// Bins of a lane in histograms of one 32-bit plane of 256 words per field.
+__device__ __forceinline__ int lane_bins(int B) { return B > 128 ? 8 : (B > 64 ? 4 : (B > 32 ? 2 : 1)); }
+
+// A lane's bpl (1, 2, 4 or 8) consecutive bins of a plane.
+__device__ __forceinline__ void ld_bins(const uint32_t* p, int bpl, uint32_t (&h)[8]) {
+#pragma unroll
+  for (int q = 0; q < 8; ++q) h[q] = 0u;
+  if (bpl >= 4) {
+    const uint4 a = reinterpret_cast<const uint4*>(p)[0];
+    h[0] = a.x, h[1] = a.y, h[2] = a.z, h[3] = a.w;
+    if (bpl == 8) {
+      const uint4 b = reinterpret_cast<const uint4*>(p)[1];
+      h[4] = b.x, h[5] = b.y, h[6] = b.z, h[7] = b.w;
+    }
+  } else if (bpl == 2) {
+    const uint2 a = *reinterpret_cast<const uint2*>(p);
+    h[0] = a.x, h[1] = a.y;
+  } else {
+    h[0] = *p;
+  }
+}
+
+__device__ __forceinline__ void st_bins(uint32_t* p, int bpl, const uint32_t (&h)[8]) {
+  if (bpl >= 4) {
+    reinterpret_cast<uint4*>(p)[0] = make_uint4(h[0], h[1], h[2], h[3]);
+    if (bpl == 8) reinterpret_cast<uint4*>(p)[1] = make_uint4(h[4], h[5], h[6], h[7]);
+  } else if (bpl == 2) {
+    *reinterpret_cast<uint2*>(p) = make_uint2(h[0], h[1]);
+  } else {
+    *p = h[0];
+  }
+}
+
+// Stable partition of a node's rows by a block: left rows in order, then right
+// rows in order.  Warp w holds in e[i] the entries of rows (w + WARPS i) 32 ..;
+// goes_left(i, r) is asked for rows below len; left: a word of shared memory
+// per 32 rows.  Returns the number of left rows.
+template <int CH, int WARPS, typename F>
+__device__ __forceinline__ uint32_t block_partition(const uint32_t (&e)[CH], uint32_t len, int64_t base, uint32_t* out,
+                                                    uint32_t* left, F&& goes_left) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t chunks = (len + 31u) / 32u;
+  unsigned bl[CH];
+#pragma unroll
+  for (int i = 0; i < CH; ++i) {
+    const uint32_t c = warp + WARPS * i, r = c * 32u + lane;
+    bl[i] = 0u;
+    if (c < chunks) {
+      bl[i] = __ballot_sync(kFull, r < len && goes_left(i, r));
+      if (lane == 0) left[c] = __popc(bl[i]);
+    }
+  }
+  __syncthreads();
+  uint32_t total = 0u, before[CH];
+#pragma unroll
+  for (int i = 0; i < CH; ++i) before[i] = 0u;
+  for (uint32_t c0 = 0; c0 < chunks; c0 += 32u) {
+    const uint32_t v = c0 + lane < chunks ? left[c0 + lane] : 0u;
+    const uint32_t x = total + warp_excl_scan_u32(v, lane);
+#pragma unroll
+    for (int i = 0; i < CH; ++i) {
+      const uint32_t c = warp + WARPS * i;
+      const uint32_t y = __shfl_sync(kFull, x, c & 31u);
+      if (c >= c0 && c < c0 + 32u) before[i] = y;
+    }
+    total = __shfl_sync(kFull, x + v, 31);
+  }
+#pragma unroll
+  for (int i = 0; i < CH; ++i) {
+    const uint32_t c = warp + WARPS * i, r = c * 32u + lane;
+    if (c < chunks && r < len) {
+      const uint32_t l = before[i] + __popc(bl[i] & lanemask_lt());
+      out[base + (((bl[i] >> lane) & 1u) ? l : total + (r - l))] = e[i];
+    }
+  }
+  return total;
+}
+
 }  // namespace
 
 }  // namespace bgb

@@ -32,7 +32,7 @@
 // bind, 17 ms at depth 11, where the scores of small nodes do.
 #include <cstdint>
 
-#include "split.cuh"
+#include "regress.cuh"
 
 namespace bgb {
 
@@ -41,65 +41,6 @@ namespace {
 constexpr int kTbWarps = 8;       // warps of a k_three_rows block
 constexpr int kTbRows = 512;      // rows staged at a time
 constexpr int kTbPitch = 136;     // words per row pair of a warp's tile (128 columns; 8 mod 32)
-
-struct RegCand {
-  float sf = -1.0f;
-  long long S = 0;
-  uint32_t nL = 0u, fb = 0xFFFFFFFFu;  // feature << 8 | threshold
-};
-
-// slot of a sampled column: the inverse permutation
-__device__ __noinline__ uint32_t perm_slot(const Perm& P, uint32_t f) {
-  if (P.n <= 1u) return f;
-  uint32_t x = f;
-  do {
-    uint32_t left = x >> P.half, right = x & P.mask;
-#pragma unroll
-    for (int r = 7; r >= 0; --r) {
-      const uint32_t prev = right ^ (murmur_fmix(left ^ P.key[r]) & P.mask);
-      right = left;
-      left = prev;
-    }
-    x = (left << P.half) | right;
-  } while (x >= P.n);
-  return x;
-}
-
-// whether candidate a comes before b, exactly (scores, then keys)
-__device__ __noinline__ bool reg_before(long long Sa, uint32_t na, uint32_t fa, long long Sb, uint32_t nb, uint32_t fb,
-                                        long long SP, uint32_t n, const Perm* P) {
-  if (fb == 0xFFFFFFFFu) return true;
-  if (!((Sa == Sb && na == nb) || (Sa == SP - Sb && na == n - nb))) {  // else the same partition
-    Cand<1> a, b;
-    make_reg<1>(a, Sa, SP, na, n);
-    make_reg<1>(b, Sb, SP, nb, n);
-    const int c = frac_cmp(a.num, a.den, b.num, b.den);
-    if (c != 0) return c > 0;
-  }
-  if (P && (fa >> 8) != (fb >> 8)) return perm_slot(*P, fa >> 8) < perm_slot(*P, fb >> 8);
-  return fa < fb;
-}
-
-// P: the node's permutation where equal scores go to the first drawn column
-__device__ __forceinline__ void reg_offer(RegCand& b, float sf, long long S, uint32_t nL, uint32_t fb, long long SP,
-                                          uint32_t n, const Perm* P) {
-  if (sf < 0.0f || sf < screen(b.sf)) return;
-  if (screen(sf) <= b.sf && !reg_before(S, nL, fb, b.S, b.nL, b.fb, SP, n, P)) return;
-  b.sf = sf;
-  b.S = S;
-  b.nL = nL;
-  b.fb = fb;
-}
-
-__device__ __forceinline__ void reg_warp_best(RegCand& b, long long SP, uint32_t n, const Perm* P) {
-#pragma unroll
-  for (int m = 1; m < 32; m <<= 1) {
-    const float sf = __shfl_xor_sync(kFull, b.sf, m);
-    const long long S = __shfl_xor_sync(kFull, b.S, m);
-    const uint32_t nL = __shfl_xor_sync(kFull, b.nL, m), fb = __shfl_xor_sync(kFull, b.fb, m);
-    reg_offer(b, sf, S, nL, fb, SP, n, P);
-  }
-}
 
 // Bits of the columns a node samples: slots first, first + step, ... by this
 // thread.
@@ -119,18 +60,6 @@ __device__ __forceinline__ void mark_columns(const Perm& P, int mtry, uint32_t f
   }
 }
 
-__device__ __forceinline__ uint32_t commit_reg(const Dev& d, uint32_t k, const RegCand& b, const NodeInfo<1>& nd) {
-  Cand<1> c;
-  c.valid = false;
-  if (b.sf >= 0.0f) {
-    make_reg<1>(c, b.S, nd.SP, b.nL, nd.n);
-    c.feat = static_cast<int32_t>(b.fb >> 8);
-    c.bin = static_cast<int32_t>(b.fb & 255u);
-    c.key = 0u;
-  }
-  return commit_split<1, 1>(d, k, c, nd);
-}
-
 // ---------------------------------------------------------------- more than 8 rows
 struct TbSmem {
   uint32_t tile[kTbWarps][8 * kTbPitch];  // [row pair][column] halves of two rows
@@ -140,19 +69,6 @@ struct TbSmem {
   Perm perm;
   uint32_t sp;
 };
-
-__device__ __forceinline__ uint32_t le_h2(uint32_t a, uint32_t b) {
-  uint32_t r;
-  asm("set.le.f16x2.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-  return r;
-}
-
-// half bits of an integer of at most 2048
-__device__ __forceinline__ uint32_t half_bits(int v) {
-  uint32_t r;
-  asm("{.reg .b16 h; cvt.rn.f16.s32 h, %1; mov.b32 %0, {h, h};}" : "=r"(r) : "r"(v));
-  return r & 0xFFFFu;
-}
 
 template <typename T>
 __device__ __forceinline__ T quad_own(const T (&p)[4], int t) {

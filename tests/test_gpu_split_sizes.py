@@ -58,3 +58,26 @@ def test_three_bin_regression(N, p, bins, discrete, tie_break):
     w = synth.Workload("t", X, y.astype(np.int64), N, p, synth.REGRESSION | synth.TREEIMP, 1, bins, 6 if N < 5000 else 2,
                        9 if N < 5000 else 2, 2, seed=N, mtry=0)
     check_iteration(w, tie_break=tie_break)
+
+
+@pytest.mark.parametrize("tie_break", [0, 1])
+@pytest.mark.parametrize("N,p,bins,mtry,target", [(13, 20, 5, 0, "plain"), (51, 20, 256, 1 << 20, "plain"),
+                                                  (60, 33, 40, 31, "wide"), (410, 12, 128, 1 << 20, "discrete"),
+                                                  (415, 20, 7, 33, "plain"), (700, 20, 200, 0, "wide"),
+                                                  (1650, 9, 256, 1 << 20, "plain"), (1700, 20, 100, 34, "discrete")])
+def test_binned_regression(N, p, bins, mtry, target, tie_break):
+    """Nodes around 8, 16, 32, 256 and 1024 rows; samples around 32 columns and
+    all of them; targets of two and of three limbs, and few distinct ones."""
+    rng = np.random.default_rng(N + p)
+    X = np.zeros((p, synth.pad16(N)), np.uint8)
+    X[:, :N] = rng.integers(0, bins, size=(p, N))
+    y = X[0, :N].astype(np.int64) - 2 * X[p // 2, :N]
+    if target == "discrete":
+        y = rng.integers(-2, 3, N) * 2**20
+    else:
+        y = y * 2**16 + rng.integers(-2**21, 2**21, N)
+    if target == "wide":
+        y = y * 2**22 - 2**44
+    w = synth.Workload("t", X, y.astype(np.int64), N, p, synth.REGRESSION | synth.TREEIMP, 1, bins, 6, 8, 2, seed=N,
+                       mtry=mtry)
+    check_iteration(w, tie_break=tie_break)
