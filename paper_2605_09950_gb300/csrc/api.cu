@@ -97,6 +97,7 @@ struct boruta_session {
   // launch geometry
   int sms = 0, split_grid = 0, small_grid = 0, tree_grid = 0, permut_grid = 0, walk_grid = 0;
   size_t split_smem = 0;
+  int col_grid = 0;             // blocks of column.cu's last kernel, 0: not for this session
   int rec_grid[3] = {0, 0, 0};  // blocks of record.cu's or threebin.cu's kernels that the GPU holds at once
   // second stream for the small-node kernel, and its fork/join events
   cudaStream_t st2 = nullptr;
@@ -440,11 +441,14 @@ static int session_init(boruta_session* s, const uint8_t* X, int64_t ld, const v
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kptr[1], kSplitThreads, s->split_smem));
   if (per_sm < 1) return fail(BORUTA_EINVAL, "split kernel does not fit on an SM");
   s->split_grid = per_sm * s->sms;
-  if (!reg)
+  if (!reg) {
     CK(static_cast<cudaError_t>(setup_record(variant, s->sms, s->rec_grid)));
-  else if (d.B <= 3)
+    CK(static_cast<cudaError_t>(setup_column(d, s->sms, &s->col_grid)));
+    if (s->col_grid > 0 && (rc = s->alloc(&d.col_cnt, p_aug_max))) return rc;
+  }
+  if (reg && d.B <= 3)
     CK(static_cast<cudaError_t>(setup_three_bins(static_cast<int>(p_aug_max), s->sms, s->rec_grid)));
-  else
+  else if (reg)
     CK(static_cast<cudaError_t>(setup_regress(s->sms, s->rec_grid)));
   // warp-per-node kernels: as many blocks as the GPU holds at once (they
   // loop over their nodes), so no partial last wave
@@ -509,6 +513,19 @@ static uint32_t record_rows(const boruta_session* s, const Dev& d) {
   return std::min<uint32_t>(kRecordRows, static_cast<uint32_t>(d.N) / (in_l2 ? 1u : 64u));
 }
 
+// Whether column.cu takes the classification nodes of more than 256 rows: the
+// columns fit in shared memory (N up to about 130,000 to 200,000, by classes).
+// Measured against record.cu and the band path (ms an iteration): N = 5003, 3
+// classes 3.34 -> 3.09; N = 30011, 8 classes 8.05 -> 6.79; N = 1e5, p = 1000
+// 141 -> 93; 12 jobs of 500 to 50,000 rows 165 -> 137.  Up to 4096 rows
+// record.cu holds every node in one launch.
+static int32_t use_columns(const boruta_session* s, const Dev& d) {
+  if (d.kind != 0 || s->split_path != 0 || s->col_grid == 0 || d.B <= 4) return 0;
+  if (d.N <= static_cast<int32_t>(kRecordRows)) return 0;
+  const uint64_t nodes = static_cast<uint64_t>(d.M) * (static_cast<uint64_t>(d.N) / 257 + 1);
+  return nodes * static_cast<uint64_t>(d.mtry) <= d.item_cap;
+}
+
 // Enqueues iteration t on the session's stream (or records it, when the
 // stream is being captured into a graph), with the copies of its status,
 // state and counters into pinned host memory; does not wait.
@@ -530,6 +547,9 @@ static int enqueue_iteration(boruta_session* s, int t, cudaStream_t st) {
   d.mtry = static_cast<int32_t>(std::max<int64_t>(m, 1));
   d.ldP = static_cast<int32_t>((p_aug + 15) / 16 * 16);
   d.rec_rows = record_rows(s, d);
+  d.columns = use_columns(s, d);
+  if (d.columns) d.rec_rows = 256;
+  const int col_grids[2] = {s->rec_grid[0], s->col_grid};
   // threebin.cu reads whole records: at most 8 times the sampled columns
   d.three_bins = d.kind == 1 && d.B <= 3 && s->split_path == 0 && s->rec_grid[0] > 0 && s->rec_grid[1] > 0 &&
                  8ll * d.mtry >= p_aug;
@@ -633,7 +653,7 @@ static int enqueue_iteration(boruta_session* s, int t, cudaStream_t st) {
     }
     s->used_bw[level] = dl.band_w;
     s->used_bl[level] = dl.band_launch;
-    nk += launch_split(dl, level, std::max(gs, 1), gi, s->rec_grid, nodes, big, s->split_smem, st, s->st2, s->fork, s->join,
+    nk += launch_split(dl, level, std::max(gs, 1), gi, d.columns ? col_grids : s->rec_grid, s->sms, nodes, big, s->split_smem, st, s->st2, s->fork, s->join,
                        timed ? s->hev[2 * level] : nullptr, timed ? s->hev[2 * level + 1] : nullptr);
     CK_LAUNCH("split kernels");
     if (timed) CK(cudaEventRecord(s->ev[2 * level + 1], st));

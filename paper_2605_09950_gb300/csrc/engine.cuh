@@ -64,6 +64,9 @@ struct Dev {
   uint32_t* nrec;                // [D + 2][3] per level: numbers of the three
   uint32_t rec2_cap;
   uint32_t rec_rows;             // largest node split by record (0: none)
+  int32_t columns;               // 1: classification nodes of more than 256 rows, weight below 65536, go to
+                                 //   column.cu (listed in rec2 from its start), rec_rows = 256
+  uint32_t* col_cnt;             // [p_aug] items per column, then their ends
   int32_t wide_y;                // regression: a row's weighted target may exceed 41 bits and its sign
   int32_t three_bins;            // 1: regression nodes below kThreeRows rows go to threebin.cu, those of at
                                  //   most 8 rows listed in `micro`, the others in `small`
@@ -135,8 +138,8 @@ int launch_bootstrap(const Dev& d, int grid, cudaStream_t st);
 // small-node kernel then runs on `st2` while the larger-node kernels run on
 // `st` (fork/join through the two events).
 // hist_start/hist_end are recorded on `st` around the histogram kernel.
-int launch_split(const Dev& d, int level, int grid_small, int grid_big, const int* grid_rec, uint64_t nodes,
-                  uint64_t big_bound, size_t smem, cudaStream_t st,
+int launch_split(const Dev& d, int level, int grid_small, int grid_big, const int* grid_rec, int sms,
+                  uint64_t nodes, uint64_t big_bound, size_t smem, cudaStream_t st,
                   cudaStream_t st2, cudaEvent_t fork, cudaEvent_t join, cudaEvent_t hist_start,
                   cudaEvent_t hist_end);
 // small.cu: the level's classification nodes of few rows, on `st`
@@ -153,6 +156,10 @@ int launch_three_bins(const Dev& d, int level, const int* grids, uint64_t nodes,
 // rows (d.rec_rows > 0), those of at most 32 on `st2`
 int setup_regress(int sms, int* grids);
 int launch_regress(const Dev& d, int level, const int* grids, uint64_t nodes, cudaStream_t st, cudaStream_t st2);
+// column.cu: whether it can take the session's columns (grid of its last
+// kernel, 0: no); the level's nodes of its list
+int setup_column(const Dev& d, int sms, int* grid);
+int launch_column(const Dev& d, int level, int sms, int finish_grid, uint64_t nodes, cudaStream_t st);
 size_t ninfo_bytes(int variant);
 int split_variant(int kind, int C);
 int variant_classes(int variant);  // largest class count of a kernel variant (1 for regression)

@@ -285,7 +285,9 @@ __global__ void __launch_bounds__(256) k_classify(Dev d, int level) {
         if (KIND == 1 && cls == 2 && nd.len <= d.rec_rows) cls = nd.len > 256u ? 7 : 6;
         if (KIND == 0 && nd.len <= kMidRows && (cls == 2 || nd.n > kFewWeight)) cls = 5;
         // by record: 10-bit counts, exact f32 products below weight 4096, 16-bit counts
-        if (KIND == 0 && cls == 2 && nd.len <= d.rec_rows && nd.n < 65536u)
+        if (KIND == 0 && cls == 2 && d.columns && nd.n < 65536u)
+          cls = nd.len <= 256u && nd.n < 1024u ? 6 : 7;
+        if (KIND == 0 && cls == 2 && !d.columns && nd.len <= d.rec_rows && nd.n < 65536u)
           cls = nd.len <= 256u && nd.n < 1024u ? 6
                 : nd.len <= 1024u && nd.n < 4096u ? (d.rec_rows > 256u ? 7 : 2)
                                                   : (d.rec_rows > 1024u ? 8 : 2);
@@ -1608,7 +1610,7 @@ __global__ void __launch_bounds__(256, BORUTA_SMALL_MINB) k_finalize(Dev d, int 
 }
 
 template <int KIND, int CM>
-int launch_level(const Dev& d, int level, int grid_small, int grid_items, const int* grid_rec, uint64_t nodes,
+int launch_level(const Dev& d, int level, int grid_small, int grid_items, const int* grid_rec, int sms, uint64_t nodes,
                  uint64_t big_bound, size_t smem, cudaStream_t st, cudaStream_t st2, cudaEvent_t fork, cudaEvent_t join, cudaEvent_t hist_start,
                  cudaEvent_t hist_end) {
   int n = 1;
@@ -1617,12 +1619,13 @@ int launch_level(const Dev& d, int level, int grid_small, int grid_items, const 
   cudaEventRecord(fork, st);
   cudaStreamWaitEvent(st2, fork, 0);
   // rows of the largest node that the kernels of the other files take
-  const uint32_t taken = KIND == 1 && d.three_bins ? kThreeRows - 1u : d.rec_rows;
+  const uint32_t taken = KIND == 1 && d.three_bins ? kThreeRows - 1u : (d.columns ? 65535u : d.rec_rows);
   const bool hist_open = taken > 0u;
   if (hist_open && hist_start) cudaEventRecord(hist_start, st);
   if constexpr (KIND == 0) {
     n += launch_few_rows(d, level, grid_small, st2);
     if (d.rec_rows > 0u) n += launch_record(d, level, grid_rec, std::max<uint64_t>(big_bound, 1), st);
+    if (d.columns) n += launch_column(d, level, sms, grid_rec[1], std::min(nodes, static_cast<uint64_t>(d.rec2_cap)), st);
   } else if (d.three_bins) {
     n += launch_three_bins(d, level, grid_rec, nodes, st, st2);
   } else if (d.rec_rows > 0u) {
@@ -1723,11 +1726,11 @@ const void* small_kernel_ptr(int variant) {
   });
 }
 
-int launch_split(const Dev& d, int level, int grid_small, int grid_big, const int* grid_rec, uint64_t nodes,
+int launch_split(const Dev& d, int level, int grid_small, int grid_big, const int* grid_rec, int sms, uint64_t nodes,
                  uint64_t big_bound, size_t smem, cudaStream_t st, cudaStream_t st2, cudaEvent_t fork, cudaEvent_t join, cudaEvent_t hs,
                  cudaEvent_t he) {
   return with_variant(split_variant(d.kind, d.C), [&](auto kind, auto cm) {
-    return launch_level<decltype(kind)::value, decltype(cm)::value>(d, level, grid_small, grid_big, grid_rec, nodes, big_bound, smem,
+    return launch_level<decltype(kind)::value, decltype(cm)::value>(d, level, grid_small, grid_big, grid_rec, sms, nodes, big_bound, smem,
                                                                      st, st2, fork, join, hs, he);
   });
 }

@@ -81,3 +81,12 @@ def test_binned_regression(N, p, bins, mtry, target, tie_break):
     w = synth.Workload("t", X, y.astype(np.int64), N, p, synth.REGRESSION | synth.TREEIMP, 1, bins, 6, 8, 2, seed=N,
                        mtry=mtry)
     check_iteration(w, tie_break=tie_break)
+
+
+@pytest.mark.parametrize("classes", [2, 3, 5, 8])
+@pytest.mark.parametrize("N,bins,mtry", [(4097, 256, 7), (5001, 33, 40), (66_000, 256, 3)])
+def test_nodes_by_column(classes, N, bins, mtry):
+    """Columns in shared memory: just above the largest tile, an odd number of
+    rows, and roots whose weight exceeds the packed counts' 16 bits."""
+    w = workload(N, 12, classes, bins, 3, 3, mtry, seed=N + classes)
+    check_iteration(w, tie_break=classes & 1)
