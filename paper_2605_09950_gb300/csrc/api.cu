@@ -253,7 +253,8 @@ static int session_init(boruta_session* s, const uint8_t* X, int64_t ld, const v
   // node pool: per tree at most min(2^l, N) nodes at depth l
   uint64_t per_tree = 0;
   for (int l = 0; l <= max_depth; ++l) per_tree += std::min<uint64_t>(1ull << l, static_cast<uint64_t>(N));
-  uint64_t cap = per_tree * static_cast<uint64_t>(n_trees);
+  // (and a place per level: its nodes start at an even index)
+  uint64_t cap = per_tree * static_cast<uint64_t>(n_trees) + static_cast<uint64_t>(max_depth) + 2;
   if (cap > 0xFFFFFFF0ull) cap = 0xFFFFFFF0ull;
   d.cap = static_cast<uint32_t>(cap);
   const int Cmax = kMaxClasses;

@@ -25,6 +25,7 @@ namespace bgb {
 namespace {
 
 constexpr unsigned kFull = 0xFFFFFFFFu;
+constexpr uint32_t kPermutNodes = 16384;  // nodes per tree up to which k_permut goes through all trees per row chunk
 
 // exclusive block scan of one u32 per thread; returns the block total in *total
 __device__ uint32_t block_excl_scan(uint32_t v, uint32_t* total, uint32_t* smem_warp) {
@@ -303,7 +304,8 @@ __global__ void k_children(Dev d, int level) {
   }
   before = block_sum<uint32_t>(before, sred);
   total = block_sum<uint32_t>(total, sred);
-  const uint32_t next_off = off + n;
+  // children start at an even index: a pair's packed words are one 16-byte load
+  const uint32_t next_off = (off + n + 1u) & ~1u;
   const uint64_t need = static_cast<uint64_t>(next_off) + 2ull * total;
   if (need > d.cap) {
     // no room for the children: the level's nodes become leaves so that every
@@ -546,13 +548,23 @@ __device__ float loss32(const Dev& d, uint32_t q, uint32_t q2) {
 // and dealt round-robin to its lanes, kWalks at a time per lane, so that a
 // lane whose row has few re-walks takes over those of a row with many.
 // Work items are (tree, chunk of 128 OOB rows), dealt round-robin to a grid
-// of exactly the blocks the GPU holds at once, so no partial last wave.
+// of exactly the blocks the GPU holds at once, so no partial last wave.  Small
+// trees: chunk by chunk through all trees, whose node words L2 holds, so that a
+// row's record is read from DRAM once for all of them (N = 1e5, 500 trees of
+// 7,000 nodes: 24.4 -> 18.9 ms).  Large trees: tree by tree, which keeps one
+// tree's nodes in L1 (N = 1e6, 300 trees of 42,000 nodes: 266 ms against 312).
 // PREC: the precision form (0 = FP64 terms, 1 = FP32 terms), a template
 // argument so that each instantiation holds one loss routine.
 __host__ __device__ inline size_t permut_smem_per_warp(int D) {
   // walk pool: start node and feature << 8 | swapped bin (32 * D each), the
   // owning lane (32 * D bytes), then each lane's row and base leaf
   return static_cast<size_t>(32 * D) * 9 + 64 * 4;
+}
+
+// The packed words of a node's two children (their pair starts at an even
+// index): one 16-byte load.
+__device__ __forceinline__ uint4 child_words(const Dev& d, uint32_t c) {
+  return *reinterpret_cast<const uint4*>(d.nd_sc + c);
 }
 
 template <int PREC>
@@ -567,12 +579,14 @@ __global__ void __launch_bounds__(128) k_permut(Dev d) {
   uint8_t* q_own = reinterpret_cast<uint8_t*>(o_leaf + 32);
   const uint32_t chunks = (static_cast<uint32_t>(d.N) + 127u) / 128u;
   const uint64_t items = static_cast<uint64_t>(d.M) * chunks;
+  const bool by_rows = (d.lvl_off[d.D] + d.lvl_cnt[d.D]) / static_cast<uint32_t>(d.M) <= kPermutNodes;
   unsigned long long visits = 0;  // nodes whose test a walk applied (the base path and the re-walks)
   constexpr int kWalks = BORUTA_PERMUT_WALKS;
   for (uint64_t item = blockIdx.x; item < items; item += gridDim.x) {
-    const int tau = static_cast<int>(item / chunks);
+    const int tau = static_cast<int>(by_rows ? item % static_cast<uint64_t>(d.M) : item / chunks);
+    const uint32_t chunk = static_cast<uint32_t>(by_rows ? item / static_cast<uint64_t>(d.M) : item % chunks);
     const uint32_t noob = d.oob_cnt[tau];
-    const uint32_t r0 = static_cast<uint32_t>(item - static_cast<uint64_t>(tau) * chunks) * 128u;
+    const uint32_t r0 = chunk * 128u;
     if (r0 >= noob) continue;  // block-uniform
     const uint32_t* oob = d.oob + static_cast<int64_t>(tau) * d.N;
     const uint32_t r = r0 + threadIdx.x;
@@ -595,15 +609,15 @@ __global__ void __launch_bounds__(128) k_permut(Dev d) {
       uint32_t s = root.x, c = root.y;
       while (depth < kMaxDepth && s != kLeaf) {
         const uint8_t x = xi[s >> 8];
-        const uint2 n0 = d.nd_sc[c], n1 = d.nd_sc[c + 1];
+        const uint4 n = child_words(d, c);
         path[depth] = k;
         pw[depth] = s;
         px[depth] = x;
         ++depth;
         const bool right = x > (s & 255u);
         k = c + (right ? 1u : 0u);
-        s = right ? n1.x : n0.x;
-        c = right ? n1.y : n0.y;
+        s = right ? n.z : n.x;
+        c = right ? n.w : n.y;
       }
       q = k;
       visits += static_cast<unsigned long long>(depth);
@@ -678,11 +692,11 @@ __global__ void __launch_bounds__(128) k_permut(Dev d) {
           const uint32_t g = ws[u] >> 8;
           const uint8_t x = (g == (fx[u] >> 8)) ? static_cast<uint8_t>(fx[u] & 255u) : xr[u][g];
           const uint32_t c = wc[u];
-          const uint2 n0 = d.nd_sc[c], n1 = d.nd_sc[c + 1];
+          const uint4 n = child_words(d, c);
           const bool right = x > (ws[u] & 255u);
           wk[u] = c + (right ? 1u : 0u);
-          ws[u] = right ? n1.x : n0.x;
-          wc[u] = right ? n1.y : n0.y;
+          ws[u] = right ? n.z : n.x;
+          wc[u] = right ? n.w : n.y;
         }
         if (!busy) break;
       }
