@@ -86,7 +86,8 @@ struct boruta_session {
   bool finished = false;
   std::vector<void*> dev_allocs;
   std::vector<int8_t> state_h;
-  // pinned staging
+  // pinned staging: one allocation
+  void* pinned = nullptr;
   uint32_t* status_h = nullptr;
   int8_t* state_pin = nullptr;
   int32_t* live_pin = nullptr;
@@ -115,17 +116,40 @@ struct boruta_session {
   cudaEvent_t iev[2] = {nullptr, nullptr};  // around the importance stage (Alg. 2 or 3)
   double imp_ms = 0.0, imp_visits = 0.0;
 
+  // Buffers of at most kSmallBytes share slabs: a session has about 45 buffers,
+  // most of them small, and each cudaMalloc / cudaFree costs microseconds and
+  // may wait for the device.
+  static constexpr size_t kSmallBytes = size_t{256} << 10, kSlabBytes = size_t{2} << 20;
+  char* slab = nullptr;
+  size_t slab_left = 0;
+
+  int raw_alloc(void** q, size_t bytes) {
+    const cudaError_t e = cudaMalloc(q, bytes);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      return fail(BORUTA_ENOMEM, "device allocation of %zu bytes failed: %s", bytes, cudaGetErrorString(e));
+    }
+    dev_allocs.push_back(*q);
+    return 0;
+  }
+
   template <typename T>
   int alloc(T** p, size_t count) {
     void* q = nullptr;
-    if (count == 0) count = 1;
-    cudaError_t e = cudaMalloc(&q, count * sizeof(T));
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      return fail(BORUTA_ENOMEM, "device allocation of %zu bytes failed: %s", count * sizeof(T),
-                  cudaGetErrorString(e));
+    const size_t bytes = (std::max<size_t>(count, 1) * sizeof(T) + 255) & ~size_t{255};
+    if (bytes > kSmallBytes) {
+      if (const int rc = raw_alloc(&q, bytes)) return rc;
+    } else {
+      if (slab_left < bytes) {
+        void* m = nullptr;
+        if (const int rc = raw_alloc(&m, kSlabBytes)) return rc;
+        slab = static_cast<char*>(m);
+        slab_left = kSlabBytes;
+      }
+      q = slab;
+      slab += bytes;
+      slab_left -= bytes;
     }
-    dev_allocs.push_back(q);
     *p = static_cast<T*>(q);
     return 0;
   }
@@ -145,11 +169,8 @@ struct boruta_session {
     if (gst) cudaStreamDestroy(gst);
     if (fork) cudaEventDestroy(fork);
     if (join) cudaEventDestroy(join);
-    if (status_h) cudaFreeHost(status_h);
-    if (counters_h) cudaFreeHost(counters_h);
+    if (pinned) cudaFreeHost(pinned);
     if (own_stream && st) cudaStreamDestroy(st);
-    if (state_pin) cudaFreeHost(state_pin);
-    if (live_pin) cudaFreeHost(live_pin);
   }
 };
 
@@ -306,10 +327,11 @@ static int session_init(boruta_session* s, const uint8_t* X, int64_t ld, const v
   if ((rc = s->alloc(&pascal, 127 * 127))) return rc;
   d.pascal = pascal;
 
-  CK(cudaHostAlloc(&s->status_h, 4 * sizeof(uint32_t), cudaHostAllocDefault));
-  CK(cudaHostAlloc(reinterpret_cast<void**>(&s->counters_h), 4 * sizeof(unsigned long long), cudaHostAllocDefault));
-  CK(cudaHostAlloc(&s->state_pin, p, cudaHostAllocDefault));
-  CK(cudaHostAlloc(&s->live_pin, p * sizeof(int32_t), cudaHostAllocDefault));
+  CK(cudaHostAlloc(&s->pinned, 64 + static_cast<size_t>(p) * (sizeof(int32_t) + 1), cudaHostAllocDefault));
+  s->counters_h = static_cast<unsigned long long*>(s->pinned);
+  s->status_h = reinterpret_cast<uint32_t*>(s->counters_h + 4);
+  s->live_pin = reinterpret_cast<int32_t*>(static_cast<char*>(s->pinned) + 64);
+  s->state_pin = reinterpret_cast<int8_t*>(s->live_pin + p);
 
   // binomial coefficients C(t, k), t, k <= 126, by Pascal's rule (exact)
   std::vector<u128> tri(127 * 127, 0);
