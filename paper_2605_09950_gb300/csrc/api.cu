@@ -438,6 +438,7 @@ static int session_init(boruta_session* s, const uint8_t* X, int64_t ld, const v
     d.frows = static_cast<uint32_t>(std::max<int64_t>(1, std::min<int64_t>(N, (int64_t{1} << 30) / per_row)));
     if (o->forest_rows > 0) d.frows = std::min<uint32_t>(d.frows, static_cast<uint32_t>(o->forest_rows));
     if ((rc = s->alloc(&d.fbase, static_cast<size_t>(N) * K * kCsaLimbs))) return rc;
+    if ((rc = s->alloc(&d.nd_value, P * K))) return rc;
     if ((rc = s->alloc(&d.fbase_mean, static_cast<size_t>(N) * K))) return rc;
     if ((rc = s->alloc(&d.facc, static_cast<size_t>(d.frows) * p_aug_max * K * kCsaLimbs))) return rc;
     CK(cudaMemsetAsync(d.facc, 0, static_cast<size_t>(d.frows) * p_aug_max * K * kCsaLimbs * sizeof(long long),

@@ -349,6 +349,39 @@ __device__ inline bool csa_add(long long* acc, double x) {
   return true;
 }
 
+// acc += a - b, exactly: the difference of the two fixed-point values in one
+// term (at most four limbs, usually three) where their lowest bits lie within
+// 32 places of each other, else the two terms.  False as csa_add.
+__device__ inline bool csa_add_diff(long long* acc, double a, double b) {
+  if (a == b) return true;
+  const uint64_t xa = static_cast<uint64_t>(__double_as_longlong(a)), xb = static_cast<uint64_t>(__double_as_longlong(b));
+  const int ea = static_cast<int>((xa >> 52) & 0x7FF), eb = static_cast<int>((xb >> 52) & 0x7FF);
+  const int pa = ea - 1075 + kFixShift, pb = eb - 1075 + kFixShift;  // places of the lowest bits
+  const int lo = pa < pb ? pa : pb;
+  if (ea == 0 || eb == 0 || ea == 0x7FF || eb == 0x7FF || lo < 0 || pa - lo > 32 || pb - lo > 32 ||
+      lo + 53 + 33 > 32 * kCsaLimbs - 2) {
+    return csa_add(acc, a) & csa_add(acc, -b);
+  }
+  const uint64_t frac = (1ull << 52) - 1ull;
+  __int128 va = static_cast<__int128>((xa & frac) | (1ull << 52)) << (pa - lo);
+  __int128 vb = static_cast<__int128>((xb & frac) | (1ull << 52)) << (pb - lo);
+  if (xa >> 63) va = -va;
+  if (xb >> 63) vb = -vb;
+  const __int128 df = va - vb;
+  const bool neg = df < 0;
+  // magnitude below 2^87: with up to 31 places to the limb's boundary, 4 chunks
+  const u128 v = static_cast<u128>(neg ? -df : df) << (lo & 31);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const uint32_t c = static_cast<uint32_t>(v >> (32 * q));
+    if (c) {
+      const long long t = neg ? -static_cast<long long>(c) : static_cast<long long>(c);
+      atomicAdd(reinterpret_cast<unsigned long long*>(acc + (lo >> 5) + q), static_cast<unsigned long long>(t));
+    }
+  }
+  return true;
+}
+
 // carry-save limbs -> 384-bit two's complement (kFixLimbs u64 limbs)
 __device__ inline void csa_to_fix(const long long* acc, uint64_t out[kFixLimbs]) {
   __int128 carry = 0;

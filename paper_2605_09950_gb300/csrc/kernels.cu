@@ -773,21 +773,37 @@ const void* permut_kernel_ptr(int precision) {
 // permuted prediction.  Each mean is that exact sum rounded once, then
 // divided by M (IEEE), and the per-row losses are summed exactly per column.
 
-__device__ __forceinline__ double leaf_value(const Dev& d, uint32_t q, int k) {
-  const double n = static_cast<double>(d.nd_n[q]);
-  return d.kind != 0 ? static_cast<double>(d.nd_S[q]) / n
-                     : static_cast<double>(d.nd_cnt[static_cast<int64_t>(q) * d.C + k]) / n;
+// Each node's value per class, divided once: the walks below read it for every
+// changed leaf, and GB300's FP64 divisions would bind them (N = 5003, 100
+// trees: 1.37 -> 0.24 ms).
+__global__ void k_leaf_values(Dev d) {
+  const int K = d.kind != 0 ? 1 : d.C;
+  const int64_t total = static_cast<int64_t>(d.lvl_off[d.D] + d.lvl_cnt[d.D]) * K;
+  for (int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; t < total;
+       t += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+    const int64_t q = t / K;
+    const int k = static_cast<int>(t - q * K);
+    const double n = static_cast<double>(d.nd_n[q]);
+    d.nd_value[t] = d.kind != 0 ? static_cast<double>(d.nd_S[q]) / n : static_cast<double>(d.nd_cnt[q * d.C + k]) / n;
+  }
 }
 
-// leaf of tree tau for row i (column f, if >= 0, read at row pi instead)
-__device__ __forceinline__ uint32_t forest_walk(const Dev& d, int tau, uint32_t i, uint32_t f, uint32_t pi) {
-  uint32_t k = static_cast<uint32_t>(tau);
-  for (int guard = 0; guard <= kMaxDepth; ++guard) {  // trees are at most kMaxDepth deep
-    const uint32_t s = d.nd_split[k];
-    if (s == kLeaf) break;
-    const uint32_t g = s >> 8;
+__device__ __forceinline__ double leaf_value(const Dev& d, uint32_t q, int k) {
+  return d.nd_value[static_cast<int64_t>(q) * (d.kind != 0 ? 1 : d.C) + k];
+}
+
+// leaf reached from node k (its packed words n) by row i, column f read at row
+// pi instead (f = 0xFFFFFFFF: none); the children's words are loaded with the
+// row's bin, one round trip a level
+__device__ __forceinline__ uint32_t forest_walk(const Dev& d, uint32_t k, uint32_t i, uint32_t f, uint32_t pi) {
+  uint2 n = d.nd_sc[k];
+  for (int guard = 0; guard <= kMaxDepth && n.x != kLeaf; ++guard) {  // trees are at most kMaxDepth deep
+    const uint32_t g = n.x >> 8;
     const uint8_t x = d.Xrow[static_cast<int64_t>(g == f ? pi : i) * d.ldP + g];
-    k = d.nd_child[k] + (x > (s & 255u) ? 1u : 0u);
+    const uint4 w = child_words(d, n.y);
+    const bool right = x > (n.x & 255u);
+    k = n.y + (right ? 1u : 0u);
+    n = right ? make_uint2(w.z, w.w) : make_uint2(w.x, w.y);
   }
   return k;
 }
@@ -802,7 +818,7 @@ __global__ void k_fperm_base(Dev d) {
        it += static_cast<int64_t>(gridDim.x) * blockDim.x) {
     const int tau = static_cast<int>(it / d.N);
     const uint32_t i = static_cast<uint32_t>(it - static_cast<int64_t>(tau) * d.N);
-    const uint32_t q = forest_walk(d, tau, i, 0xFFFFFFFFu, 0u);
+    const uint32_t q = forest_walk(d, static_cast<uint32_t>(tau), i, 0xFFFFFFFFu, 0u);
     for (int k = 0; k < K; ++k)
       if (!csa_add(d.fbase + (static_cast<int64_t>(i) * K + k) * kCsaLimbs, leaf_value(d, q, k)))
         atomicOr(&d.status[0], kErrAcc);
@@ -834,13 +850,22 @@ __global__ void k_fperm_delta(Dev d, uint32_t r0, uint32_t rows) {
     const uint32_t loc = static_cast<uint32_t>(it - static_cast<int64_t>(tau) * rows);
     const uint32_t i = r0 + loc;
     const uint32_t pi = d.piv[i];
-    uint32_t pw[kMaxDepth];
+    // the row's path: split words, children and the row's own bins
+    uint32_t pw[kMaxDepth], pc[kMaxDepth];
+    uint8_t px[kMaxDepth];
     int depth = 0;
     uint32_t k = static_cast<uint32_t>(tau);
-    for (uint32_t s = d.nd_split[k]; s != kLeaf && depth < kMaxDepth; s = d.nd_split[k]) {
-      const uint8_t x = d.Xrow[static_cast<int64_t>(i) * d.ldP + (s >> 8)];
-      pw[depth++] = s;
-      k = d.nd_child[k] + (x > (s & 255u) ? 1u : 0u);
+    uint2 n = d.nd_sc[k];
+    while (n.x != kLeaf && depth < kMaxDepth) {
+      const uint8_t x = d.Xrow[static_cast<int64_t>(i) * d.ldP + (n.x >> 8)];
+      const uint4 w = child_words(d, n.y);
+      pw[depth] = n.x;
+      pc[depth] = n.y;
+      px[depth] = x;
+      ++depth;
+      const bool right = x > (n.x & 255u);
+      k = n.y + (right ? 1u : 0u);
+      n = right ? make_uint2(w.z, w.w) : make_uint2(w.x, w.y);
     }
     const uint32_t q = k;
     for (int a = 0; a < depth; ++a) {  // a column off the path leaves the leaf unchanged
@@ -848,14 +873,18 @@ __global__ void k_fperm_delta(Dev d, uint32_t r0, uint32_t rows) {
       bool seen = false;
       for (int b = 0; b < a; ++b) seen |= (pw[b] >> 8) == f;
       if (seen) continue;
-      const uint32_t q2 = forest_walk(d, tau, i, f, pi);
+      // the first node on the path that tests f and sends the swapped value the other way
+      const uint8_t xp = d.Xrow[static_cast<int64_t>(pi) * d.ldP + f];
+      int b = a;
+      for (; b < depth; ++b)
+        if ((pw[b] >> 8) == f && ((xp > (pw[b] & 255u)) != (px[b] > (pw[b] & 255u)))) break;
+      if (b == depth) continue;  // the same leaf
+      const uint32_t q2 = forest_walk(d, pc[b] + ((xp > (pw[b] & 255u)) ? 1u : 0u), i, f, pi);
       if (q2 == q) continue;
       long long* acc = d.facc + ((static_cast<int64_t>(loc) * d.p_aug + f) * K) * kCsaLimbs;
       bool ok = true;
-      for (int c = 0; c < K; ++c) {
-        ok &= csa_add(acc + c * kCsaLimbs, leaf_value(d, q2, c));
-        ok &= csa_add(acc + c * kCsaLimbs, -leaf_value(d, q, c));
-      }
+      for (int c = 0; c < K; ++c)
+        ok &= csa_add_diff(acc + c * kCsaLimbs, leaf_value(d, q2, c), leaf_value(d, q, c));
       if (!ok) atomicOr(&d.status[0], kErrAcc);
     }
   }
@@ -912,10 +941,12 @@ __global__ void k_fperm_final(Dev d) {
 int launch_forest_permut(const Dev& d, int grid, cudaStream_t st) {
   int n = 0;
   k_permut_pi<<<(d.N + 255) / 256 < 1024 ? (d.N + 255) / 256 : 1024, 256, 0, st>>>(d);
+  k_pack_nodes<<<grid, 256, 0, st>>>(d);
+  k_leaf_values<<<grid, 256, 0, st>>>(d);
   cudaMemsetAsync(d.fbase, 0, static_cast<size_t>(d.N) * forest_k(d) * kCsaLimbs * sizeof(long long), st);
   k_fperm_base<<<grid, 256, 0, st>>>(d);
   k_fperm_base_mean<<<grid, 256, 0, st>>>(d);
-  n += 3;
+  n += 5;
   for (uint32_t r0 = 0; r0 < static_cast<uint32_t>(d.N); r0 += d.frows) {
     const uint32_t rows = min(d.frows, static_cast<uint32_t>(d.N) - r0);
     k_fperm_delta<<<grid, 256, 0, st>>>(d, r0, rows);
