@@ -368,7 +368,9 @@ static int session_init(boruta_session* s, const uint8_t* X, int64_t ld, const v
   d.B = std::max(2, std::min(n_bins, static_cast<int>(s->status_h[3]) + 1));
   if (reg) {
     d.C = 1;
-    d.wide_y = maxy >= (1ull << 33);  // 255 maxy: 41 bits and a sign (regress.cu)
+    // a row's weighted target (at most 255 maxy) in 41 bits and a sign, and any
+    // sum of them below 2^53 (regress.cu, threebin.cu, score_reg_narrow)
+    d.wide_y = maxy >= (1ull << 33) || static_cast<double>(maxy) * static_cast<double>(N) >= 9007199254740992.0;
     if (maxy && static_cast<double>(maxy) * static_cast<double>(N) >= 4611686018427387904.0)
       return fail(BORUTA_EOVERFLOW, "N * max|y| must stay below 2^62");
   } else {

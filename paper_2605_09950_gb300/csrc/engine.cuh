@@ -67,7 +67,8 @@ struct Dev {
   int32_t columns;               // 1: classification nodes of more than 256 rows, weight below 65536, go to
                                  //   column.cu (listed in rec2 from its start), rec_rows = 256
   uint32_t* col_cnt;             // [p_aug] items per column, then their ends
-  int32_t wide_y;                // regression: a row's weighted target may exceed 41 bits and its sign
+  int32_t wide_y;                // regression: a row's weighted target may exceed 41 bits and its sign, or a
+                                 //   sum of them 2^53
   int32_t three_bins;            // 1: regression nodes below kThreeRows rows go to threebin.cu, those of at
                                  //   most 8 rows listed in `micro`, the others in `small`
   uint32_t small_cap;            // entries of `small`

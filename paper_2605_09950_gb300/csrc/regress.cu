@@ -21,7 +21,7 @@
 // Every lane keeps its best candidate exactly (regress.cuh).
 //
 // Measured: N = 10000, p = 50, all 100 columns tried, 100 trees, depth 16,
-// 128 bins: 26.4 -> 17.7 ms an iteration (row-by-row sums through shuffles and
+// 128 bins: 26.4 -> 16.1 ms an iteration (row-by-row sums through shuffles and
 // 64-bit shared-memory atomics before).
 #include <algorithm>
 #include <cstdint>
@@ -119,7 +119,7 @@ __device__ void reg_few(const Dev& d, int level, uint32_t k, RegWarp& sm, unsign
     long long S;
     uint32_t nL;
     subset(m, S, nL);
-    sm.few.score[m] = nL > 0u && nL < nd.n ? score_reg_f(S, nd.SP, nL, nd.n) : -1.0f;
+    sm.few.score[m] = nL > 0u && nL < nd.n ? score_reg_any(d.wide_y, S, nd.SP, nL, nd.n) : -1.0f;
   }
   __syncwarp();
   RegCand best;
@@ -142,15 +142,25 @@ __device__ void reg_few(const Dev& d, int level, uint32_t k, RegWarp& sm, unsign
         if (b[r] <= b[s]) m[s] |= 1u << r;
       }
     }
+    // the candidates that may come first (few), their subsets and bins by byte
+    uint32_t cand = 0u;
+    unsigned long long ms = 0ull, xs = 0ull;
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
       if (r >= len) break;
       const float sf = sm.few.score[m[r]];
-      if (!in || sf < 0.0f || sf < screen(best.sf)) continue;
+      if (in && sf >= 0.0f && sf >= screen(best.sf)) cand |= 1u << r;
+      ms |= static_cast<unsigned long long>(m[r]) << (8 * r);
+      xs |= static_cast<unsigned long long>(b[r]) << (8 * r);
+    }
+    for (; cand; cand &= cand - 1u) {
+      const int r = __ffs(cand) - 1;
+      const uint32_t sub = static_cast<uint32_t>(ms >> (8 * r)) & 255u;
       long long S;
       uint32_t nL;
-      subset(m[r], S, nL);
-      reg_offer(best, sf, S, nL, key_of(d, j, f) | b[r], nd.SP, nd.n, nullptr);
+      subset(sub, S, nL);
+      reg_offer(best, sm.few.score[sub], S, nL, key_of(d, j, f) | (static_cast<uint32_t>(xs >> (8 * r)) & 255u), nd.SP,
+                nd.n, nullptr);
     }
   }
   reg_warp_best(best, nd.SP, nd.n, nullptr);
@@ -276,14 +286,13 @@ __device__ void reg_rows(const Dev& d, int level, uint32_t k, RegWarp& sm, unsig
       const int a0 = o ? m[1] : m[0], a1 = o ? m[3] : m[2];
       const int p2 = __shfl_xor_sync(kFull, h ? a0 : a1, 2), p3 = __shfl_xor_sync(kFull, h ? x0 : x1, 2);
       const int p0 = h ? a1 : a0, p1 = h ? x1 : x0;  // of lanes t, t ^ 1; p2, p3: of t ^ 2, t ^ 3
-      auto part = [&](int p, int lane_t) {
-        return lane_t == 3 ? 0ll : static_cast<long long>(static_cast<unsigned long long>(static_cast<long long>(p))
-                                                          << (22 * lane_t));
-      };
-      const long long S = part(p0, t) + part(p1, t ^ 1) + part(p2, t ^ 2) + part(p3, t ^ 3);
-      const uint32_t nL = static_cast<uint32_t>(t == 3 ? p0 : (t == 2 ? p1 : (t == 1 ? p2 : p3)));
+      const int u0 = o ? p1 : p0, u1 = o ? p0 : p1, u2 = o ? p3 : p2, u3 = o ? p2 : p3;
+      const int v0 = h ? u2 : u0, v1 = h ? u3 : u1, v2 = h ? u0 : u2, v3 = h ? u1 : u3;  // of lanes 0..3
+      const long long S = static_cast<long long>(v0) + static_cast<long long>(v1) * (1ll << 22) +
+                          static_cast<long long>(static_cast<unsigned long long>(static_cast<long long>(v2)) << 44);
+      const uint32_t nL = static_cast<uint32_t>(v3);
       if (own && nL < n_own)
-        reg_offer(best, score_reg_f(S, SP_own, nL, n_own), S, nL,
+        reg_offer(best, score_reg_any(d.wide_y, S, SP_own, nL, n_own), S, nL,
                   key_of(d, r0 + j, sm.feat[sseg][r0 + j]) | th[8 * t + g], SP_own, n_own, nullptr);
     }
   }
@@ -440,7 +449,7 @@ __device__ __forceinline__ void reg_record(const Dev& d, int level, uint32_t k, 
         nL += h[0][q];
         S += bs[q];
         if (nL < nd.n)
-          reg_offer(best, score_reg_f(S, nd.SP, nL, nd.n), S, nL, key | static_cast<uint32_t>(lane * bpl + q), nd.SP,
+          reg_offer(best, score_reg_any(d.wide_y, S, nd.SP, nL, nd.n), S, nL, key | static_cast<uint32_t>(lane * bpl + q), nd.SP,
                     nd.n, nullptr);
       }
       const uint32_t zero[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};

@@ -87,6 +87,7 @@ __device__ void three_rows(const Dev& d, int level, uint32_t k, TbSmem& sm, uint
   const uint32_t len = nd.len, words = (static_cast<uint32_t>(d.p_aug) + 31u) / 32u;
   for (uint32_t i = threadIdx.x; i < words; i += kTbWarps * 32) bits[i] = 0u;
   if (threadIdx.x == 0) node_perm(d, k, sm.perm);
+  const bool short_sums = !d.wide_y && len < 4096u;  // five limbs (45 bits and a sign) and 32-bit partial sums
   auto stage = [&](uint32_t r0) {  // rows r0 .. of the node
     const uint32_t nr = min(static_cast<uint32_t>(kTbRows), (len - r0 + 15u) & ~15u);
     for (uint32_t i = threadIdx.x; i < nr; i += kTbWarps * 32) {
@@ -97,8 +98,11 @@ __device__ void three_rows(const Dev& d, int level, uint32_t k, TbSmem& sm, uint
       const long long x = v ? static_cast<long long>(w) * d.yreg[e >> 8] : 0ll;
       uint16_t* h = reinterpret_cast<uint16_t*>(&sm.val[i >> 1][0]) + (i & 1u);
 #pragma unroll
-      for (int j = 0; j < 6; ++j) h[2 * j] = static_cast<uint16_t>(half_bits(static_cast<int>((x >> (9 * j)) & 511)));
-      h[12] = static_cast<uint16_t>(half_bits(static_cast<int>(x >> 54)));
+      for (int j = 0; j < 6; ++j) {
+        const int limb = static_cast<int>((x >> (9 * j)) & 511);
+        h[2 * j] = static_cast<uint16_t>(half_bits(short_sums && j >= 4 ? (j == 4 ? static_cast<int>(x >> 36) : 0) : limb));
+      }
+      h[12] = static_cast<uint16_t>(half_bits(short_sums ? 0 : static_cast<int>(x >> 54)));
       h[14] = static_cast<uint16_t>(half_bits(static_cast<int>(w)));
     }
     return nr;
@@ -168,23 +172,47 @@ __device__ void three_rows(const Dev& d, int level, uint32_t k, TbSmem& sm, uint
     // two column groups at a time: lane t of a quad takes group t / 2, threshold t % 2
 #pragma unroll
     for (int q = 0; q < 16; q += 2) {
-      long long part[4];
-      uint32_t cnt[4];
+      long long S;
+      uint32_t nL;
+      if (!short_sums) {
+        long long part[4];
+        uint32_t cnt[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int m0 = __float_as_int(acc[q + (i >> 1)][2 * (i & 1)] + bias) - ibias;
-        const int m1 = __float_as_int(acc[q + (i >> 1)][2 * (i & 1) + 1] + bias) - ibias;
-        // (modulo 2^64: the total fits)
-        part[i] = static_cast<long long>(
-            static_cast<unsigned long long>(static_cast<long long>(m0) + (t == 3 ? 0ll : 512ll * m1)) << (18 * t));
-        cnt[i] = t == 3 ? static_cast<uint32_t>(m1) : 0u;
+        for (int i = 0; i < 4; ++i) {
+          const int m0 = __float_as_int(acc[q + (i >> 1)][2 * (i & 1)] + bias) - ibias;
+          const int m1 = __float_as_int(acc[q + (i >> 1)][2 * (i & 1) + 1] + bias) - ibias;
+          // (modulo 2^64: the total fits)
+          part[i] = static_cast<long long>(
+              static_cast<unsigned long long>(static_cast<long long>(m0) + (t == 3 ? 0ll : 512ll * m1)) << (18 * t));
+          cnt[i] = t == 3 ? static_cast<uint32_t>(m1) : 0u;
+        }
+        S = quad_own(part, t);
+        nL = quad_own(cnt, t);
+      } else {
+        // limbs 0..4, the last one signed (its lane's other column is 0), and the
+        // weight: a lane's two columns in 32 bits (rows < 4096), transposed over
+        // the quad
+        int m[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int m0 = __float_as_int(acc[q + (i >> 1)][2 * (i & 1)] + 12582912.0f) - 0x4B400000;
+          const int m1 = __float_as_int(acc[q + (i >> 1)][2 * (i & 1) + 1] + 12582912.0f) - 0x4B400000;
+          m[i] = t == 3 ? m1 : m0 + (m1 << 9);
+        }
+        const bool o = t & 1, h = t & 2;
+        const int x0 = __shfl_xor_sync(kFull, o ? m[0] : m[1], 1), x1 = __shfl_xor_sync(kFull, o ? m[2] : m[3], 1);
+        const int a0 = o ? m[1] : m[0], a1 = o ? m[3] : m[2];
+        const int p2 = __shfl_xor_sync(kFull, h ? a0 : a1, 2), p3 = __shfl_xor_sync(kFull, h ? x0 : x1, 2);
+        const int p0 = h ? a1 : a0, p1 = h ? x1 : x0;  // of lanes t, t ^ 1; p2, p3: of t ^ 2, t ^ 3
+        const int u0 = o ? p1 : p0, u1 = o ? p0 : p1, u2 = o ? p3 : p2, u3 = o ? p2 : p3;
+        const int v0 = h ? u2 : u0, v1 = h ? u3 : u1, v2 = h ? u0 : u2, v3 = h ? u1 : u3;  // of lanes 0..3
+        S = static_cast<long long>(v0) + (static_cast<long long>(v1) << 18) + static_cast<long long>(v2) * (1ll << 36);
+        nL = static_cast<uint32_t>(v3);
       }
-      const long long S = quad_own(part, t);
-      const uint32_t nL = quad_own(cnt, t);
       const uint32_t f = f0 + 8u * (q + (t >> 1)) + g;
       const bool drawn = f < static_cast<uint32_t>(d.p_aug) && ((bits[f >> 5] >> (f & 31u)) & 1u);
       if (drawn && nL > 0u && nL < nd.n)
-        reg_offer(best, score_reg_f(S, nd.SP, nL, nd.n), S, nL, (f << 8) | static_cast<uint32_t>(t & 1), nd.SP, nd.n,
+        reg_offer(best, score_reg_any(d.wide_y, S, nd.SP, nL, nd.n), S, nL, (f << 8) | static_cast<uint32_t>(t & 1), nd.SP, nd.n,
                   order);
     }
   }
@@ -258,7 +286,7 @@ __device__ void three_few(const Dev& d, int level, uint32_t k, TbFew& sm, uint32
     long long S;
     uint32_t nL;
     subset(m, S, nL);
-    sm.score[m] = nL > 0u && nL < nd.n ? score_reg_f(S, nd.SP, nL, nd.n) : -1.0f;
+    sm.score[m] = nL > 0u && nL < nd.n ? score_reg_any(d.wide_y, S, nd.SP, nL, nd.n) : -1.0f;
   }
   mark_columns(P, d.mtry, static_cast<uint32_t>(lane), 32u, bits);
   __syncwarp();
