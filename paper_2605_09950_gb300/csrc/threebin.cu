@@ -27,9 +27,9 @@
 // so the chosen split is that of an exhaustive exact comparison.
 //
 // Measured: N = 20000, p = 5003, 100 trees, depth 12, a third of the columns
-// sampled: 556 -> 105 ms an iteration (gathers of columns and warp reductions
-// before); 5.4 to 6.9 ms a level down to depth 7, where the 12.6 GB of records
-// bind, 17 ms at depth 11, where the scores of small nodes do.
+// sampled: 556 -> 88 ms an iteration (gathers of columns and warp reductions
+// before); about 6 ms a level down to depth 7, 13.5 ms at depth 11.  Bound by
+// the ALU pipe (62% busy at depth 10): bytes to half pairs, comparisons, scores.
 #include <cstdint>
 
 #include "regress.cuh"
@@ -169,51 +169,61 @@ __device__ void three_rows(const Dev& d, int level, uint32_t k, TbSmem& sm, uint
       }
     }
     if (!mine) continue;
+    if (short_sums) {
+      // Limbs 0..4 (the last one signed; its lane's other column is 0) and the
+      // weight: a lane's two columns in 32 bits (rows < 4096).  The quads' parts
+      // go through the tile, so that the lanes then score the sampled columns
+      // only, one after another.
+      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < 16; ++q)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+          const int m0 = __float_as_int(acc[q][2 * b] + 12582912.0f) - 0x4B400000;
+          const int m1 = __float_as_int(acc[q][2 * b + 1] + 12582912.0f) - 0x4B400000;
+          tile[((8 * q + g) * 2 + b) * 4 + t] = static_cast<uint32_t>(t == 3 ? m1 : m0 + (m1 << 9));
+        }
+      uint8_t* list = reinterpret_cast<uint8_t*>(tile + 1024);  // the block's sampled columns
+      uint32_t count = 0u;
+#pragma unroll
+      for (uint32_t w = 0; w < 4; ++w) {
+        const uint32_t bw = (f0 >> 5) + w < words ? bits[(f0 >> 5) + w] : 0u;
+        if ((bw >> lane) & 1u) list[count + __popc(bw & lanemask_lt())] = static_cast<uint8_t>(32u * w + lane);
+        count += __popc(bw);
+      }
+      __syncwarp();
+      for (uint32_t i = lane; i < 2u * count; i += 32u) {
+        const uint32_t c = list[i >> 1], b = i & 1u;
+        const int4 m = reinterpret_cast<const int4*>(tile)[2u * c + b];
+        const long long S = static_cast<long long>(m.x) + (static_cast<long long>(m.y) << 18) +
+                            static_cast<long long>(m.z) * (1ll << 36);
+        const uint32_t nL = static_cast<uint32_t>(m.w);
+        if (nL > 0u && nL < nd.n)
+          reg_offer(best, score_reg_narrow(S, nd.SP, nL, nd.n), S, nL, ((f0 + c) << 8) | b, nd.SP, nd.n, order);
+      }
+      continue;
+    }
     // two column groups at a time: lane t of a quad takes group t / 2, threshold t % 2
 #pragma unroll
     for (int q = 0; q < 16; q += 2) {
-      long long S;
-      uint32_t nL;
-      if (!short_sums) {
-        long long part[4];
-        uint32_t cnt[4];
+      long long part[4];
+      uint32_t cnt[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int m0 = __float_as_int(acc[q + (i >> 1)][2 * (i & 1)] + bias) - ibias;
-          const int m1 = __float_as_int(acc[q + (i >> 1)][2 * (i & 1) + 1] + bias) - ibias;
-          // (modulo 2^64: the total fits)
-          part[i] = static_cast<long long>(
-              static_cast<unsigned long long>(static_cast<long long>(m0) + (t == 3 ? 0ll : 512ll * m1)) << (18 * t));
-          cnt[i] = t == 3 ? static_cast<uint32_t>(m1) : 0u;
-        }
-        S = quad_own(part, t);
-        nL = quad_own(cnt, t);
-      } else {
-        // limbs 0..4, the last one signed (its lane's other column is 0), and the
-        // weight: a lane's two columns in 32 bits (rows < 4096), transposed over
-        // the quad
-        int m[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int m0 = __float_as_int(acc[q + (i >> 1)][2 * (i & 1)] + 12582912.0f) - 0x4B400000;
-          const int m1 = __float_as_int(acc[q + (i >> 1)][2 * (i & 1) + 1] + 12582912.0f) - 0x4B400000;
-          m[i] = t == 3 ? m1 : m0 + (m1 << 9);
-        }
-        const bool o = t & 1, h = t & 2;
-        const int x0 = __shfl_xor_sync(kFull, o ? m[0] : m[1], 1), x1 = __shfl_xor_sync(kFull, o ? m[2] : m[3], 1);
-        const int a0 = o ? m[1] : m[0], a1 = o ? m[3] : m[2];
-        const int p2 = __shfl_xor_sync(kFull, h ? a0 : a1, 2), p3 = __shfl_xor_sync(kFull, h ? x0 : x1, 2);
-        const int p0 = h ? a1 : a0, p1 = h ? x1 : x0;  // of lanes t, t ^ 1; p2, p3: of t ^ 2, t ^ 3
-        const int u0 = o ? p1 : p0, u1 = o ? p0 : p1, u2 = o ? p3 : p2, u3 = o ? p2 : p3;
-        const int v0 = h ? u2 : u0, v1 = h ? u3 : u1, v2 = h ? u0 : u2, v3 = h ? u1 : u3;  // of lanes 0..3
-        S = static_cast<long long>(v0) + (static_cast<long long>(v1) << 18) + static_cast<long long>(v2) * (1ll << 36);
-        nL = static_cast<uint32_t>(v3);
+      for (int i = 0; i < 4; ++i) {
+        const int m0 = __float_as_int(acc[q + (i >> 1)][2 * (i & 1)] + bias) - ibias;
+        const int m1 = __float_as_int(acc[q + (i >> 1)][2 * (i & 1) + 1] + bias) - ibias;
+        // (modulo 2^64: the total fits)
+        part[i] = static_cast<long long>(
+            static_cast<unsigned long long>(static_cast<long long>(m0) + (t == 3 ? 0ll : 512ll * m1)) << (18 * t));
+        cnt[i] = t == 3 ? static_cast<uint32_t>(m1) : 0u;
       }
+      const long long S = quad_own(part, t);
+      const uint32_t nL = quad_own(cnt, t);
       const uint32_t f = f0 + 8u * (q + (t >> 1)) + g;
       const bool drawn = f < static_cast<uint32_t>(d.p_aug) && ((bits[f >> 5] >> (f & 31u)) & 1u);
       if (drawn && nL > 0u && nL < nd.n)
-        reg_offer(best, score_reg_any(d.wide_y, S, nd.SP, nL, nd.n), S, nL, (f << 8) | static_cast<uint32_t>(t & 1), nd.SP, nd.n,
-                  order);
+        reg_offer(best, score_reg_any(d.wide_y, S, nd.SP, nL, nd.n), S, nL, (f << 8) | static_cast<uint32_t>(t & 1),
+                  nd.SP, nd.n, order);
     }
   }
   reg_warp_best(best, nd.SP, nd.n, order);
