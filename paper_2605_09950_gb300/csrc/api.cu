@@ -683,7 +683,7 @@ static int enqueue_iteration(boruta_session* s, int t, cudaStream_t st) {
                        timed ? s->hev[2 * level] : nullptr, timed ? s->hev[2 * level + 1] : nullptr);
     CK_LAUNCH("split kernels");
     if (timed) CK(cudaEventRecord(s->ev[2 * level + 1], st));
-    nk += launch_children(d, level, st);
+    nk += launch_children(d, level, nodes, st);
     CK_LAUNCH("next-level kernels");
   }
   if (timed) CK(cudaEventRecord(s->iev[0], st));

@@ -170,7 +170,7 @@ const void* small_kernel_ptr(int variant);  // for its occupancy
 size_t cand_bytes(int variant);
 size_t packed_bytes(int variant);
 int launch_gather_live(const Dev& d, cudaStream_t st);
-int launch_children(const Dev& d, int level, cudaStream_t st);
+int launch_children(const Dev& d, int level, uint64_t nodes, cudaStream_t st);
 int launch_treeimp(const Dev& d, int grid, cudaStream_t st);
 int launch_permut(const Dev& d, int grid, int walk_grid, cudaStream_t st);
 // Xrow (the row-major copy of Xaug): built once per iteration, after the

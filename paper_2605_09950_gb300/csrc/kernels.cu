@@ -14,7 +14,7 @@
 // synchronous); node work is claimed dynamically by persistent CTAs.
 #include <cstdint>
 
-#include "engine.cuh"
+#include "lists.cuh"
 
 #ifndef BORUTA_PERMUT_WALKS
 #define BORUTA_PERMUT_WALKS 8  // re-walks of one OOB row advanced together
@@ -291,16 +291,28 @@ __global__ void k_count(Dev d, int level) {
   if (threadIdx.x == 0) d.chunk[blockIdx.x] = tot;
 }
 
-__global__ void k_children(Dev d, int level) {
+// The children also go to the next level's lists.  self: the blocks count the
+// level's splits themselves (few nodes: less than a k_count launch).
+__global__ void k_children(Dev d, int level, int self) {
   __shared__ uint32_t sw[33];
   __shared__ uint32_t sred[256];
   const uint32_t n = d.lvl_cnt[level], off = d.lvl_off[level];
   const uint32_t chunk = (n + gridDim.x - 1) / gridDim.x;
   uint32_t before = 0, total = 0;
-  for (uint32_t b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
-    const uint32_t v = d.chunk[b];
-    total += v;
-    before += b < blockIdx.x ? v : 0u;
+  if (self) {
+    const uint32_t start = blockIdx.x * chunk;
+#pragma unroll 8
+    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
+      const uint32_t v = d.nd_split[off + i] != kLeaf ? 1u : 0u;
+      total += v;
+      before += i < start ? v : 0u;
+    }
+  } else {
+    for (uint32_t b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
+      const uint32_t v = d.chunk[b];
+      total += v;
+      before += b < blockIdx.x ? v : 0u;
+    }
   }
   before = block_sum<uint32_t>(before, sred);
   total = block_sum<uint32_t>(total, sred);
@@ -333,6 +345,8 @@ __global__ void k_children(Dev d, int level) {
     const bool sp = i < hi && d.nd_split[k] != kLeaf;
     uint32_t tot;
     const uint32_t r = block_excl_scan(sp ? 1u : 0u, &tot, sw);
+    int cls_l = 0, cls_r = 0;
+    uint32_t child = 0u;
     if (sp) {
       const uint32_t L = next_off + 2u * (run + r), R = L + 1u;
       d.nd_child[k] = L;
@@ -348,6 +362,7 @@ __global__ void k_children(Dev d, int level) {
       d.nd_len[R] = len - lrows;
       d.nd_n[L] = ln;
       d.nd_n[R] = n_ - ln;
+      bool pure_l = false, pure_r = false;
       if (reg) {
         const long long sl = d.nd_lS[k];
         d.nd_S[L] = sl;
@@ -356,9 +371,15 @@ __global__ void k_children(Dev d, int level) {
         for (int c = 0; c < C; ++c) {
           const uint32_t lc = d.nd_lcnt[static_cast<int64_t>(k) * C + c];
           d.nd_cnt[static_cast<int64_t>(L) * C + c] = lc;
-          d.nd_cnt[static_cast<int64_t>(R) * C + c] = d.nd_cnt[static_cast<int64_t>(k) * C + c] - lc;
+          const uint32_t rc = d.nd_cnt[static_cast<int64_t>(k) * C + c] - lc;
+          d.nd_cnt[static_cast<int64_t>(R) * C + c] = rc;
+          pure_l |= lc == ln;
+          pure_r |= rc == n_ - ln;
         }
       }
+      child = L;
+      if (lrows >= 2u && !pure_l) cls_l = node_class(d, lrows, ln);
+      if (len - lrows >= 2u && !pure_r) cls_r = node_class(d, len - lrows, n_ - ln);
       d.nd_split[L] = kLeaf;
       d.nd_split[R] = kLeaf;
       d.nd_child[L] = 0u;
@@ -366,13 +387,22 @@ __global__ void k_children(Dev d, int level) {
       d.nd_delta[L] = 0.0;
       d.nd_delta[R] = 0.0;
     }
+    if (level + 1 < d.D) {
+      list_node(d, level + 1, cls_l, child);
+      list_node(d, level + 1, cls_r, child + 1u);
+    }
     run += tot;
   }
 }
 
-int launch_children(const Dev& d, int level, cudaStream_t st) {
+// nodes: at most so many at the level
+int launch_children(const Dev& d, int level, uint64_t nodes, cudaStream_t st) {
+  if (nodes <= 16384u) {
+    k_children<<<static_cast<unsigned>((nodes + 511u) / 512u), 256, 0, st>>>(d, level, 1);
+    return 1;
+  }
   k_count<<<kScanBlocks, 256, 0, st>>>(d, level);
-  k_children<<<kScanBlocks, 256, 0, st>>>(d, level);
+  k_children<<<kScanBlocks, 256, 0, st>>>(d, level, 0);
   return 2;
 }
 

@@ -3,8 +3,8 @@
 // TreeImp accumulators (Alg. 2) and the stable row partition.
 //
 // Kernels of a level:
-//   k_classify      leaves, and the lists of small (<= 32 rows) and larger
-//                   active nodes.
+//   k_classify      (first level) leaves, and the lists of active nodes; the
+//                   other levels' lists come with their nodes (k_children).
 //   k_split_small   (second stream) one warp per node of at most 32 rows:
 //                   one row per lane, left class counts from ballots over the
 //                   bin bits against weight and class bit planes (regression:
@@ -35,6 +35,7 @@
 #include <cstdint>
 #include <type_traits>
 
+#include "lists.cuh"
 #include "split.cuh"
 
 // resident CTAs per SM the kernels are compiled for (register budget)
@@ -262,59 +263,24 @@ __device__ void small_feature(const NodeInfo<CM>& nd, int C, int B, bool v, uint
   if (take && better(c, best)) best = c;
 }
 
-// One thread per node of the level: leaves are marked, active nodes are
-// listed as micro (<= 8 rows, in `micro`), tiny (9..16 rows, from the end of
-// `small`), small (17..32 rows, from its start), mid (classification: 33..64
-// rows, or fewer with a weight above kFewWeight) or larger (warp-aggregated
-// appends).
+// The lists of the first level, one thread per root: leaves are marked, active
+// nodes listed.  (The later levels' lists are written with their nodes.)
 template <int KIND, int CM>
 __global__ void __launch_bounds__(256) k_classify(Dev d, int level) {
-  const int lane = threadIdx.x & 31;
   const uint32_t lcount = d.lvl_cnt[level], loff = d.lvl_off[level];
   for (uint32_t base = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; base < lcount;
        base += gridDim.x * blockDim.x) {
-    const uint32_t idx = base + lane;
-    int cls = 0;  // 0 none, 1 small, 2 larger, 3 tiny, 4 micro, 5 mid, 6..8 by record
-    uint32_t k = 0;
+    const uint32_t idx = base + (threadIdx.x & 31u);
+    int cls = 0;
+    const uint32_t k = loff + idx;
     if (idx < lcount) {
-      k = loff + idx;
       NodeInfo<CM> nd;
-      if (load_node<KIND, CM>(d, k, level, nd)) {
-        cls = nd.len > kFewRows ? 2 : (nd.len > 16u ? 1 : (nd.len > 8u ? 3 : 4));
-        if (KIND == 1 && d.three_bins) cls = nd.len >= kThreeRows ? 2 : (nd.len > 8u ? 1 : 4);
-        if (KIND == 1 && cls == 2 && nd.len <= d.rec_rows) cls = nd.len > 256u ? 7 : 6;
-        if (KIND == 0 && nd.len <= kMidRows && (cls == 2 || nd.n > kFewWeight)) cls = 5;
-        // by record: 10-bit counts, exact f32 products below weight 4096, 16-bit counts
-        if (KIND == 0 && cls == 2 && d.columns && nd.n < 65536u)
-          cls = nd.len <= 256u && nd.n < 1024u ? 6 : 7;
-        if (KIND == 0 && cls == 2 && !d.columns && nd.len <= d.rec_rows && nd.n < 65536u)
-          cls = nd.len <= 256u && nd.n < 1024u ? 6
-                : nd.len <= 1024u && nd.n < 4096u ? (d.rec_rows > 256u ? 7 : 2)
-                                                  : (d.rec_rows > 1024u ? 8 : 2);
-      } else {
+      if (load_node<KIND, CM>(d, k, level, nd))
+        cls = node_class(d, nd.len, nd.n);
+      else
         d.nd_split[k] = kLeaf;
-      }
     }
-    auto append = [&](int c, uint32_t* count) {
-      const unsigned m = __ballot_sync(kFull, cls == c);
-      uint32_t at = 0;
-      if (lane == 0 && m) at = atomicAdd(count, static_cast<uint32_t>(__popc(m)));
-      return __shfl_sync(kFull, at, 0) + __popc(m & lanemask_lt());
-    };
-    const uint32_t s0 = append(1, &d.nsmall[level]), b0 = append(2, &d.work[level]), t0 = append(3, &d.ntiny[level]),
-                   m0 = append(4, &d.nmicro[level]), d0 = KIND == 0 ? append(5, &d.nmid[level]) : 0u;
-    if (cls == 1) d.small[s0] = k;
-    if (cls == 2) d.big[b0] = k;
-    if (cls == 3) d.small[d.small_cap - 1u - t0] = k;
-    if (cls == 4) d.micro[m0] = k;
-    if (cls == 5) d.mid[d0] = k;
-    if (d.rec_rows > 0u) {
-      const uint32_t r0 = append(6, &d.nrec[3 * level]), r1 = append(7, &d.nrec[3 * level + 1]),
-                     r2 = append(8, &d.nrec[3 * level + 2]);
-      if (cls == 6) d.rec[r0] = k;
-      if (cls == 7) d.rec2[r1] = k;
-      if (cls == 8) d.rec2[d.rec2_cap - 1u - r2] = k;
-    }
+    list_node(d, level, cls, k);
   }
 }
 
@@ -1613,8 +1579,11 @@ template <int KIND, int CM>
 int launch_level(const Dev& d, int level, int grid_small, int grid_items, const int* grid_rec, int sms, uint64_t nodes,
                  uint64_t big_bound, size_t smem, cudaStream_t st, cudaStream_t st2, cudaEvent_t fork, cudaEvent_t join, cudaEvent_t hist_start,
                  cudaEvent_t hist_end) {
-  int n = 1;
-  k_classify<KIND, CM><<<grid_small, 256, 0, st>>>(d, level);
+  int n = 0;
+  if (level == 0) {
+    k_classify<KIND, CM><<<grid_small, 256, 0, st>>>(d, level);
+    ++n;
+  }
   // small nodes on st2, concurrently with the larger-node kernels on st
   cudaEventRecord(fork, st);
   cudaStreamWaitEvent(st2, fork, 0);
