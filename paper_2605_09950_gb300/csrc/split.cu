@@ -5,10 +5,11 @@
 // Kernels of a level:
 //   k_classify      (first level) leaves, and the lists of active nodes; the
 //                   other levels' lists come with their nodes (k_children).
-//   k_split_small   (second stream) one warp per node of at most 32 rows:
-//                   one row per lane, left class counts from ballots over the
-//                   bin bits against weight and class bit planes (regression:
-//                   shuffles, or warp reductions for columns of <= 4 bins).
+//   small.cu, record.cu, column.cu, regress.cu, threebin.cu take the nodes
+//   that their kernels are made for (lists.cuh); here:
+//   k_split_small   (second stream) regression nodes of at most 32 rows that
+//                   the others leave: one row per lane, left sums by shuffles,
+//                   or warp reductions for columns of at most 4 bins.
 //   larger nodes, feature-band path (default), in chunks of nodes whose
 //   items fit the plan buffers:
 //     k_plan_gen / k_plan_scan / k_plan_scatter  the nodes' (node, draw slot)
@@ -16,9 +17,9 @@
 //                   in, cut into (node, band) groups sorted by band, so that
 //                   the columns being gathered at any moment fit in L2;
 //     k_items_band  one warp per group: per feature a warp-private
-//                   shared-memory histogram (entries of nodes of <= 64 rows
-//                   staged once per group; class weights packed 12 bits
-//                   each into one 64-bit word per bin when they fit), a
+//                   shared-memory histogram (entries of regression nodes of
+//                   <= 64 rows staged once per group; class weights packed 12
+//                   bits each into one 64-bit word per bin when they fit), a
 //                   float pre-screen over the non-empty bins, and the
 //                   feature's exact best candidate, kept as the integers
 //                   that define it;
@@ -59,15 +60,6 @@ namespace {
 constexpr int kSmallAhead = BORUTA_SMALL_AHEAD;
 
 // ============================================================ small nodes
-// Bit planes of a small node's rows (one row per lane): the valid lanes, the
-// five bits of each row's weight and, per class, the lanes of that class.
-template <int CM>
-struct SmallPlanes {
-  unsigned valid;
-  unsigned w[5];
-  unsigned y[CM];
-};
-
 // A small node's rows sit one per lane in a segment of SEG lanes: the whole
 // warp (SEG = 32, nodes of 17..32 rows), a half warp (SEG = 16: two nodes of
 // 9..16 rows per warp) or a quarter warp (SEG = 8: four nodes of <= 8 rows).
@@ -105,10 +97,10 @@ __device__ __forceinline__ long long seg_sum_i64(long long v) {
 
 // best of the segment's lane candidates flagged valid (all lanes take part;
 // each segment walks its own candidates, as many rounds as the busier one)
-template <int KIND, int CM, int SEG>
-__device__ void seg_select(const Cand<CM>& mine, Cand<CM>& out) {
+template <int SEG>
+__device__ void seg_select(const Cand<1>& mine, Cand<1>& out) {
   if (SEG == 32) {
-    warp_select<KIND, CM>(mine, out);
+    warp_select<1, 1>(mine, out);
     return;
   }
   unsigned m = __ballot_sync(kFull, mine.valid) & seg_mask<SEG>();
@@ -118,7 +110,7 @@ __device__ void seg_select(const Cand<CM>& mine, Cand<CM>& out) {
     const bool have = m != 0u;
     const int l = have ? __ffs(m) - 1 : static_cast<int>(threadIdx.x & 31);
     if (have) m &= m - 1;
-    Cand<CM> c;
+    Cand<1> c;
     c.num.w[0] = __shfl_sync(kFull, mine.num.w[0], l);
     c.num.w[1] = __shfl_sync(kFull, mine.num.w[1], l);
     c.num.w[2] = __shfl_sync(kFull, mine.num.w[2], l);
@@ -127,35 +119,25 @@ __device__ void seg_select(const Cand<CM>& mine, Cand<CM>& out) {
     c.nL = __shfl_sync(kFull, mine.nL, l);
     c.feat = __shfl_sync(kFull, mine.feat, l);
     c.bin = __shfl_sync(kFull, mine.bin, l);
-    if (KIND == 1) {
-      c.SL = __shfl_sync(kFull, mine.SL, l);
-#pragma unroll
-      for (int k = 0; k < CM; ++k) c.cL[k] = 0u;
-    } else {
-      c.SL = 0;
-#pragma unroll
-      for (int k = 0; k < CM; ++k) c.cL[k] = __shfl_sync(kFull, mine.cL[k], l);
-    }
+    c.SL = __shfl_sync(kFull, mine.SL, l);
+    c.cL[0] = 0u;
     c.valid = have;
     if (better(c, out)) out = c;
   }
 }
 
-// Best split of one feature for a node of <= SEG rows, one row per lane of
-// its segment.  Classification: the lanes whose bin is <= this lane's bin
-// come from eight ballots over the bin bits (most significant first), and
-// the left class counts from population counts against the weight and class
-// bit planes.  Regression: the left sums are accumulated over the rows by
-// shuffles (rows up to lenmax, the longest node of the warp; lanes past a
-// node's rows carry weight 0).  Updates the node's exact best (best) and
-// best float score so far (bestf).  Every lane runs every warp-wide step:
-// a segment with nothing to contribute goes on with no candidate.
-template <int KIND, int CM, int SEG>
-__device__ void small_feature(const NodeInfo<CM>& nd, int C, int B, bool v, uint32_t b, uint32_t w, uint32_t y,
-                              long long yv, const SmallPlanes<CM>& pl, int feat, uint32_t tkey, float& bestf,
-                              Cand<CM>& best, uint32_t lenmax) {
+// Best split of one feature for a regression node of <= SEG rows, one row per
+// lane of its segment: the left sums are accumulated over the rows by shuffles
+// (rows up to lenmax, the longest node of the warp; lanes past a node's rows
+// carry weight 0), or, for columns of at most 4 bins, by reductions per
+// threshold.  Updates the node's exact best (best) and best float score so far
+// (bestf).  Every lane runs every warp-wide step: a segment with nothing to
+// contribute goes on with no candidate.
+template <int SEG>
+__device__ void small_feature(const NodeInfo<1>& nd, int B, bool v, uint32_t b, uint32_t w, long long yv, int feat,
+                              uint32_t tkey, float& bestf, Cand<1>& best, uint32_t lenmax) {
   const unsigned sm = seg_mask<SEG>();
-  if (KIND == 1 && B <= 4) {
+  if (B <= 4) {
     // Regression on a column of at most 4 bins: the left sums of each of
     // the <= 3 thresholds come from segment reductions, the same on every
     // lane of the segment.  A threshold whose bin holds no row repeats the
@@ -186,8 +168,8 @@ __device__ void small_feature(const NodeInfo<CM>& nd, int C, int B, bool v, uint
 #pragma unroll
     for (int t = 0; t < 3; ++t) {
       if (sf[t] < 0.0f || sf[t] < thr) continue;
-      Cand<CM> c;
-      make_reg<CM>(c, SLt[t], nd.SP, nLt[t], nd.n);
+      Cand<1> c;
+      make_reg<1>(c, SLt[t], nd.SP, nLt[t], nd.n);
       c.feat = feat;
       c.bin = t;
       c.key = (tkey << 8) | static_cast<uint32_t>(t);
@@ -195,49 +177,21 @@ __device__ void small_feature(const NodeInfo<CM>& nd, int C, int B, bool v, uint
     }
     return;
   }
-  uint32_t cl[CM];
-#pragma unroll
-  for (int k = 0; k < CM; ++k) cl[k] = 0u;
   uint32_t nL = 0;
   long long SL = 0;
-  unsigned same;
-  if (KIND == 0) {
-    unsigned lt = 0u, eq = pl.valid & sm;
-#pragma unroll
-    for (int t = 7; t >= 0; --t) {
-      const unsigned bt = __ballot_sync(kFull, (b >> t) & 1u);
-      const bool one = (b >> t) & 1u;
-      lt |= one ? (eq & ~bt) : 0u;
-      eq &= one ? bt : ~bt;
+  const int base = static_cast<int>(threadIdx.x & 31) & ~(SEG - 1);
+  for (int j = 0; j < static_cast<int>(lenmax); ++j) {
+    const uint32_t bj = __shfl_sync(kFull, b, base + j), wj = __shfl_sync(kFull, w, base + j);
+    const long long yj = __shfl_sync(kFull, yv, base + j);
+    if (bj <= b) {  // rows past the node's own carry weight 0
+      nL += wj;
+      SL += static_cast<long long>(wj) * yj;
     }
-    const unsigned le = lt | eq;
-#pragma unroll
-    for (int k = 0; k < CM; ++k)
-      if (k < C) {
-        const unsigned m = le & pl.y[k];
-        uint32_t c = 0;
-#pragma unroll
-        for (int t = 0; t < 5; ++t) c += static_cast<uint32_t>(__popc(m & pl.w[t])) << t;
-        cl[k] = c;
-        nL += c;
-      }
-    same = v ? eq : 0u;
-  } else {
-    const int base = static_cast<int>(threadIdx.x & 31) & ~(SEG - 1);
-    for (int j = 0; j < static_cast<int>(lenmax); ++j) {
-      const uint32_t bj = __shfl_sync(kFull, b, base + j), wj = __shfl_sync(kFull, w, base + j);
-      const long long yj = __shfl_sync(kFull, yv, base + j);
-      if (bj <= b) {  // rows past the node's own carry weight 0
-        nL += wj;
-        SL += static_cast<long long>(wj) * yj;
-      }
-    }
-    same = __match_any_sync(kFull, v ? b : 0xFFFFFFFFu) & sm;
   }
+  const unsigned same = __match_any_sync(kFull, v ? b : 0xFFFFFFFFu) & sm;
   // lanes holding the same bin propose the same partition: the lowest one speaks
   const bool ok = v && nL < nd.n && (__ffs(same) - 1) == static_cast<int>(threadIdx.x & 31);
-  float sf = -1.0f;
-  if (ok) sf = KIND == 1 ? score_reg_f(SL, nd.SP, nL, nd.n) : score_class_f<CM>(cl, nd.cp, C, nL, nd.n);
+  const float sf = ok ? score_reg_f(SL, nd.SP, nL, nd.n) : -1.0f;
   const float mx = seg_max_f<SEG>(sf);
   // a feature whose best float score is below the window of the node's best
   // so far cannot hold the node's exact best
@@ -247,19 +201,16 @@ __device__ void small_feature(const NodeInfo<CM>& nd, int C, int B, bool v, uint
     thr = screen(fmaxf(mx, bestf));
     bestf = fmaxf(mx, bestf);
   }
-  Cand<CM> mine;
+  Cand<1> mine;
   mine.valid = false;
   if (take && ok && sf >= thr) {
-    if (KIND == 1)
-      make_reg<CM>(mine, SL, nd.SP, nL, nd.n);
-    else
-      make_class<CM>(mine, cl, nd.cp, C, nL, nd.n);
+    make_reg<1>(mine, SL, nd.SP, nL, nd.n);
     mine.feat = feat;
     mine.bin = static_cast<int32_t>(b);
     mine.key = (tkey << 8) | b;
   }
-  Cand<CM> c;
-  seg_select<KIND, CM, SEG>(mine, c);
+  Cand<1> c;
+  seg_select<SEG>(mine, c);
   if (take && better(c, best)) best = c;
 }
 
@@ -288,39 +239,30 @@ constexpr uint32_t kNoNode = 0xFFFFFFFFu;
 
 // The split of the small node k of this lane's segment (kNoNode: none; its
 // lanes still take part in every warp-wide step), its record and partition.
-template <int KIND, int CM, int SEG>
+template <int SEG>
 __device__ void small_node(const Dev& d, int level, uint32_t k, uint8_t* sbin, unsigned long long& bytes) {
   const int lane = threadIdx.x & 31;
   const int hl = lane & (SEG - 1);
   const uint32_t* rows_in = d.rows[level & 1];
   uint32_t* rows_out = d.rows[(level & 1) ^ 1];
-  const int C = ncls<CM>(d);
   const bool has = k != kNoNode;
-  NodeInfo<CM> nd;
+  NodeInfo<1> nd;
   nd.base = 0;
   nd.len = 0u;
   nd.n = 0u;
   nd.SP = 0;
-#pragma unroll
-  for (int c = 0; c < CM; ++c) nd.cp[c] = 0u;
+  nd.cp[0] = 0u;
   Perm P;
   if (has) {
-    load_node<KIND, CM>(d, k, level, nd);
+    load_node<1, 1>(d, k, level, nd);
     node_perm(d, k, P);
   }
   const bool v = hl < static_cast<int>(nd.len);
   const uint32_t e = v ? rows_in[nd.base + hl] : 0u;
-  const uint32_t row = e >> 8, w = v ? ent_w<KIND>(e) : 0u;
-  const uint32_t y = KIND == 0 ? ent_y(e) : 0u;
-  const long long yv = (KIND == 1 && v) ? d.yreg[row] : 0ll;
-  SmallPlanes<CM> pl;
-  pl.valid = __ballot_sync(kFull, v);
-#pragma unroll
-  for (int t = 0; t < 5; ++t) pl.w[t] = __ballot_sync(kFull, (w >> t) & 1u);
-#pragma unroll
-  for (int c = 0; c < CM; ++c) pl.y[c] = __ballot_sync(kFull, v && y == static_cast<uint32_t>(c));
+  const uint32_t row = e >> 8, w = v ? ent_w<1>(e) : 0u;
+  const long long yv = v ? d.yreg[row] : 0ll;
   const uint32_t lenmax = SEG == 32 ? nd.len : __reduce_max_sync(kFull, nd.len);
-  Cand<CM> best;
+  Cand<1> best;
   best.valid = false;
   float bestf = -1.0f;
   for (int r0 = 0; r0 < d.mtry; r0 += SEG) {
@@ -344,15 +286,14 @@ __device__ void small_node(const Dev& d, int level, uint32_t k, uint8_t* sbin, u
       for (int u = 0; u < nu; ++u) {
         const uint32_t f = __shfl_sync(kFull, myf, j0 + u, SEG);
         const uint32_t tkey = d.tie_break == 1 ? static_cast<uint32_t>(r0 + j0 + u) : f;
-        small_feature<KIND, CM, SEG>(nd, C, d.B, v, sbin[u * 32 + lane], w, y, yv, pl, static_cast<int>(f), tkey,
-                                     bestf, best, lenmax);
+        small_feature<SEG>(nd, d.B, v, sbin[u * 32 + lane], w, yv, static_cast<int>(f), tkey, bestf, best, lenmax);
       }
     }
   }
   uint32_t sp = kLeaf;
-  if (has && hl == 0) sp = commit_split<KIND, CM>(d, k, best, nd);
+  if (has && hl == 0) sp = commit_split<1, 1>(d, k, best, nd);
   sp = __shfl_sync(kFull, sp, 0, SEG);
-  if (has && hl == 0) bytes += static_cast<unsigned long long>(nd.len) * (d.mtry + 4ull + (KIND ? 8ull : 0ull));
+  if (has && hl == 0) bytes += static_cast<unsigned long long>(nd.len) * (d.mtry + 12ull);
   // stable partition: left rows in order, then right rows in order
   const bool split = has && sp != kLeaf;
   const uint32_t bs = (v && split) ? row_bin(d, row, sp >> 8) : 0u;
@@ -370,8 +311,9 @@ __device__ void small_node(const Dev& d, int level, uint32_t k, uint8_t* sbin, u
 
 // SEG = 8: one warp per four micro nodes (a quarter warp each); SEG = 16:
 // one warp per pair of tiny nodes (a half warp each); SEG = 32: one warp per
-// small node.
-template <int KIND, int CM, int SEG>
+// small node.  Regression nodes that regress.cu and threebin.cu do not take
+// (more than kRegColumns sampled columns, four bins, split_path = 1).
+template <int SEG>
 __global__ void __launch_bounds__(256, BORUTA_SMALL_MINB) k_split_small(Dev d, int level) {
   __shared__ uint8_t sbins[8][kSmallAhead * 32];
   const int lane = threadIdx.x & 31;
@@ -384,18 +326,18 @@ __global__ void __launch_bounds__(256, BORUTA_SMALL_MINB) k_split_small(Dev d, i
     for (uint32_t idx = gwarp; idx < nquads; idx += nwarps) {
       const uint32_t t = 4u * idx + static_cast<uint32_t>(lane >> 3);
       const uint32_t k = t < nm ? d.micro[t] : kNoNode;
-      small_node<KIND, CM, SEG>(d, level, k, sbin, bytes);
+      small_node<SEG>(d, level, k, sbin, bytes);
     }
   } else if (SEG == 16) {
     const uint32_t nt = d.ntiny[level], npairs = (nt + 1u) / 2u;
     for (uint32_t idx = gwarp; idx < npairs; idx += nwarps) {
       const uint32_t t = 2u * idx + static_cast<uint32_t>(lane >> 4);
       const uint32_t k = t < nt ? d.small[d.small_cap - 1u - t] : kNoNode;
-      small_node<KIND, CM, SEG>(d, level, k, sbin, bytes);
+      small_node<SEG>(d, level, k, sbin, bytes);
     }
   } else {
     const uint32_t ns_nodes = d.nsmall[level];
-    for (uint32_t idx = gwarp; idx < ns_nodes; idx += nwarps) small_node<KIND, CM, SEG>(d, level, d.small[idx], sbin, bytes);
+    for (uint32_t idx = gwarp; idx < ns_nodes; idx += nwarps) small_node<SEG>(d, level, d.small[idx], sbin, bytes);
   }
   if (bytes) atomicAdd(&d.counters[0], bytes);
 }
@@ -926,19 +868,6 @@ __device__ void build_hist_pk(int64_t base, uint32_t len, const uint32_t* rows, 
   __syncwarp();
 }
 
-// Packed histogram of one feature over a staged node (entries in ebuf, the
-// feature's bins gathered into b; the histogram is zero on entry).
-__device__ __forceinline__ void hist_staged_pk(uint32_t len, const uint32_t* ebuf, const uint32_t (&b)[kRegRows / 32],
-                                               unsigned long long* hp) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int q = 0; q < static_cast<int>(kRegRows / 32); ++q) {
-    const uint32_t r = q * 32 + lane;
-    if (r < len) atomicAdd(&hp[b[q] + (b[q] >> 3)], pk_entry(ebuf[r]));
-  }
-  __syncwarp();
-}
-
 // Exact best among a packed histogram's candidates whose float score is at
 // least thr (several lie inside the screen window: rare, so kept out of line).
 // cand: the lane's candidate bins to revisit; pre: the warp prefix before them.
@@ -1055,17 +984,16 @@ __device__ void scan_pack_pk(const Dev& d, const NodeInfo<CM>& nd, unsigned long
   __syncwarp();
 }
 
-// Histogram of one feature over a node of at most kRegRows rows whose entries
+// Histogram of one feature over a regression node of at most kRegRows rows whose entries
 // are staged in the warp's shared memory (ebuf), the feature's bins already
 // gathered into b (lane l holds rows q * 32 + l).
 // The histogram is all zero on entry (the staged path leaves it so, see
 // hist_unstage); the bins that receive rows are marked in occ.
-template <int KIND>
 __device__ __forceinline__ void hist_staged(const Dev& d, uint32_t len, const uint32_t* ebuf,
                                             const uint32_t (&b)[kRegRows / 32], uint32_t* hw, uint32_t* occ,
                                             bool mark) {
   const int lane = threadIdx.x & 31;
-  if (regs4(d, KIND)) {
+  if (regs4(d, 1)) {
     if (lane == 0 && mark) occ[0] = (1u << d.B) - 1u;  // regs4_store writes bins 0..B-1
     uint32_t c0[4] = {0u, 0u, 0u, 0u}, c1[4] = {0u, 0u, 0u, 0u};
     long long sy[4] = {0, 0, 0, 0};
@@ -1074,35 +1002,23 @@ __device__ __forceinline__ void hist_staged(const Dev& d, uint32_t len, const ui
       const uint32_t r = q * 32 + lane;
       const bool v = r < len;
       const uint32_t e = v ? ebuf[r] : 0u;
-      regs4_add<KIND>(b[q], e, v, (KIND == 1 && v) ? d.yreg[e >> 8] : 0ll, c0, c1, sy);
+      regs4_add<1>(b[q], e, v, v ? d.yreg[e >> 8] : 0ll, c0, c1, sy);
     }
-    regs4_store<KIND>(d, hw, c0, c1, sy);
+    regs4_store<1>(d, hw, c0, c1, sy);
     return;
   }
-  if (KIND == 0) {
+  uint32_t* hn = hw;
+  unsigned long long* hs = reinterpret_cast<unsigned long long*>(hw + hist_words_n(d.B));
 #pragma unroll
-    for (int q = 0; q < static_cast<int>(kRegRows / 32); ++q) {
-      const uint32_t r = q * 32 + lane;
-      if (r < len) {
-        const uint32_t e = ebuf[r];
-        atomicAdd(&hw[b[q] * d.C + ent_y(e) + (b[q] >> 3)], ent_w<0>(e));
-        if (mark) atomicOr(&occ[b[q] >> 5], 1u << (b[q] & 31u));
-      }
-    }
-  } else {
-    uint32_t* hn = hw;
-    unsigned long long* hs = reinterpret_cast<unsigned long long*>(hw + hist_words_n(d.B));
-#pragma unroll
-    for (int q = 0; q < static_cast<int>(kRegRows / 32); ++q) {
-      const uint32_t r = q * 32 + lane;
-      if (r < len) {
-        const uint32_t e = ebuf[r];
-        const uint32_t w = ent_w<1>(e);
-        const long long yq = d.yreg[e >> 8];
-        atomicAdd(&hn[b[q] + (b[q] >> 3)], w);
-        atomicAdd(&hs[b[q] + (b[q] >> 3)], static_cast<unsigned long long>(static_cast<long long>(w) * yq));
-        if (mark) atomicOr(&occ[b[q] >> 5], 1u << (b[q] & 31u));
-      }
+  for (int q = 0; q < static_cast<int>(kRegRows / 32); ++q) {
+    const uint32_t r = q * 32 + lane;
+    if (r < len) {
+      const uint32_t e = ebuf[r];
+      const uint32_t w = ent_w<1>(e);
+      const long long yq = d.yreg[e >> 8];
+      atomicAdd(&hn[b[q] + (b[q] >> 3)], w);
+      atomicAdd(&hs[b[q] + (b[q] >> 3)], static_cast<unsigned long long>(static_cast<long long>(w) * yq));
+      if (mark) atomicOr(&occ[b[q] >> 5], 1u << (b[q] & 31u));
     }
   }
   __syncwarp();
@@ -1118,19 +1034,14 @@ __device__ __forceinline__ uint32_t lane_occ(const Dev& d, const uint32_t* occ) 
 
 // Zeroes the occupied bins of a staged histogram (each lane its own, after
 // its own reads) and the bitmap, so that the next feature starts from zero.
-template <int KIND>
 __device__ __forceinline__ void hist_unstage(const Dev& d, uint32_t* hw, uint32_t* occ, uint32_t mine) {
   const int lane = threadIdx.x & 31;
   const int bpl = (d.B + 31) >> 5;
   const int b0 = lane * bpl;
   for (uint32_t m = mine; m; m &= m - 1) {
     const int bb = b0 + __ffs(m) - 1;
-    if (KIND == 0) {
-      for (int k = 0; k < d.C; ++k) hw[bb * d.C + k + (bb >> 3)] = 0u;
-    } else {
-      hw[bb + (bb >> 3)] = 0u;
-      reinterpret_cast<unsigned long long*>(hw + hist_words_n(d.B))[bb + (bb >> 3)] = 0ull;
-    }
+    hw[bb + (bb >> 3)] = 0u;
+    reinterpret_cast<unsigned long long*>(hw + hist_words_n(d.B))[bb + (bb >> 3)] = 0ull;
   }
   __syncwarp();
   if (lane < 9) occ[lane] = 0u;
@@ -1358,7 +1269,7 @@ __global__ void __launch_bounds__(kSplitThreads, BORUTA_ITEMS_MINB) k_items_band
     // warp's shared-memory buffer, for all the group's features, and the
     // next feature's bins are gathered while this one's are counted and
     // scanned.  Larger nodes stream their entries per feature.
-    const bool staged = len <= kRegRows;
+    const bool staged = KIND == 1 && len <= kRegRows;  // (smaller classification nodes are not in this list)
     uint32_t ev[kRegRows / 32];
     if (staged) {
       const uint32_t* src = rows_in + static_cast<int64_t>(gb >> 24);
@@ -1399,18 +1310,11 @@ __global__ void __launch_bounds__(kSplitThreads, BORUTA_ITEMS_MINB) k_items_band
         if (j + 1 < count)
           gather_staged(column(d, static_cast<uint32_t>(__shfl_sync(kFull, chunk, (j + 1) & 31) & 0x3FFFFFu)),
                         nd.len, ebuf, bn);
-        if constexpr (KIND == 0 && CM <= 5) {
-          if (pk) {
-            hist_staged_pk(nd.len, ebuf, b, hp);
-            scan_pack_pk<CM>(d, nd, hp, f, dst);
-            continue;
-          }
-        }
-        hist_staged<KIND>(d, nd.len, ebuf, b, hw, occ, sparse);
+        hist_staged(d, nd.len, ebuf, b, hw, occ, sparse);
         if (sparse) {
           const uint32_t mine = lane_occ(d, occ);
           scan_pack<KIND, CM>(d, nd, hw, f, out + (static_cast<uint32_t>(it >> 22) & 0x3FFFu), mine);
-          hist_unstage<KIND>(d, hw, occ, mine);
+          hist_unstage(d, hw, occ, mine);
         } else {
           scan_pack<KIND, CM>(d, nd, hw, f, out + (static_cast<uint32_t>(it >> 22) & 0x3FFFu));
           __syncwarp();
@@ -1600,9 +1504,9 @@ int launch_level(const Dev& d, int level, int grid_small, int grid_items, const 
   } else if (d.rec_rows > 0u) {
     n += launch_regress(d, level, grid_rec, nodes, st, st2);
   } else {
-    k_split_small<KIND, CM, 8><<<grid_small, 256, 0, st2>>>(d, level);
-    k_split_small<KIND, CM, 16><<<grid_small, 256, 0, st2>>>(d, level);
-    k_split_small<KIND, CM, 32><<<grid_small, 256, 0, st2>>>(d, level);
+    k_split_small<8><<<grid_small, 256, 0, st2>>>(d, level);
+    k_split_small<16><<<grid_small, 256, 0, st2>>>(d, level);
+    k_split_small<32><<<grid_small, 256, 0, st2>>>(d, level);
     n += 3;
   }
   cudaEventRecord(join, st2);
