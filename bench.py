@@ -497,7 +497,8 @@ def run_gpu(args):
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak if peak else None, "traffic": traffic,
                      "traffic_source": prof["profile"] if traffic else None,
-                     "kernel": "k_items_band (feature histograms + exact scan of the larger nodes)",
+                     "kernel": "split kernels of the nodes of more than 64 rows (k_record, k_column, k_items_band; "
+                               "regression: k_reg_record, k_three_rows, k_items_band)",
                      "peak_kind": f"{peak_kind} hbm_gbs (burst copy)", "launches": int(ks["launches"]),
                      "kernel_ms_per_step": ks["hist_ms"] / args.steps,
                      "algorithmic_bytes_per_launch": ks["hist_bytes"] / max(1, ks["launches"]),

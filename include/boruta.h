@@ -70,8 +70,9 @@ typedef struct {
   int graph;       /* 1: each iteration is captured into a CUDA graph and replayed through one
                       executable graph, updated in place from iteration to iteration (same
                       results; per-level kernel times are then not recorded) */
-  int split_path;  /* larger nodes: 0 = feature-band-sorted groups, in chunks of nodes (default),
-                      1 = grouped items only; results are identical */
+  int split_path;  /* nodes that are split by column gathers (larger than the by-record,
+                      by-column and few-row kernels take): 0 = feature-band-sorted groups, in
+                      chunks of nodes (default), 1 = grouped items only; results are identical */
   int chunk_nodes; /* band path: at most this many larger nodes per chunk (0 = as many as the
                       plan buffers hold, the default); results are identical whatever the value,
                       a small value runs the multi-chunk path on small problems */
@@ -85,7 +86,8 @@ typedef struct {
                       many as fit in about 1 GiB, the default); results are identical */
   int autotune;    /* 1: the first step of a session (of every job of a batch) times its
                       iteration once per histogram tile shape, restoring the state after each,
-                      and keeps the fastest: column bytes per feature band (12, 24, 48, 96,
+                      and keeps the fastest (the shapes concern the nodes that are split by
+                      column gathers): column bytes per feature band (12, 24, 48, 96,
                       192 MiB) x one histogram launch per chunk of nodes or per band, and a
                       single band (no band order), at 8192 row-feature work per group of a
                       larger node, each run also timing every tree level; then the per-level
@@ -248,13 +250,16 @@ int boruta_session_dump(boruta_session* s, int what, void* host, int64_t capacit
 
 /* Timing of the last step, from CUDA events on the session's stream (any
  * pointer may be NULL):
- *   hist_ms, hist_bytes  the histogram kernel of the larger nodes (per tree
- *                        level): total milliseconds and the method's
- *                        algorithmic bytes -- one bin per (row, sampled
+ *   hist_ms, hist_bytes  the histogram kernels of the larger nodes (more
+ *                        than 64 rows in classification, more than 8 to 32
+ *                        in regression; per tree level, their scans and
+ *                        partitions included where one launch does them):
+ *                        total milliseconds and the method's algorithmic
+ *                        bytes -- one bin per (row, sampled
  *                        feature) pair plus the row's state once per node
  *                        (entry read and rewritten, weight and label: 10 B;
  *                        17 B with the 8-byte regression target)
- *   launches             number of tree levels (histogram-kernel launches)
+ *   launches             number of tree levels
  *   split_ms, split_bytes the whole split stage of the levels (classify,
  *                        histograms, split records, partition), and its
  *                        algorithmic bytes (bins per (row, feature) pair, row
