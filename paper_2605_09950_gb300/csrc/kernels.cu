@@ -387,10 +387,7 @@ __global__ void k_children(Dev d, int level, int self) {
       d.nd_delta[L] = 0.0;
       d.nd_delta[R] = 0.0;
     }
-    if (level + 1 < d.D) {
-      list_node(d, level + 1, cls_l, child);
-      list_node(d, level + 1, cls_r, child + 1u);
-    }
+    if (level + 1 < d.D) list_pair(d, level + 1, cls_l, cls_r, child);
     run += tot;
   }
 }

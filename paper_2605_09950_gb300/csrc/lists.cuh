@@ -28,25 +28,18 @@ __device__ __forceinline__ int node_class(const Dev& d, uint32_t len, uint32_t n
                                      : (d.rec_rows > 1024u ? 8 : 2);
 }
 
-// Appends node k to the level's list of its class (0: none); all lanes of the
-// warp together, one atomic per class and warp, all classes' at once.
-__device__ __forceinline__ void list_node(const Dev& d, int level, int cls, uint32_t k) {
-  const int lane = static_cast<int>(threadIdx.x & 31u);
-  const unsigned same = __match_any_sync(0xFFFFFFFFu, cls);
-  const int leader = __ffs(static_cast<int>(same)) - 1;
-  uint32_t* count = nullptr;
+__device__ __forceinline__ uint32_t* list_count(const Dev& d, int level, int cls) {
   switch (cls) {
-    case 1: count = &d.nsmall[level]; break;
-    case 2: count = &d.work[level]; break;
-    case 3: count = &d.ntiny[level]; break;
-    case 4: count = &d.nmicro[level]; break;
-    case 5: count = &d.nmid[level]; break;
-    case 6: case 7: case 8: count = &d.nrec[3 * level + cls - 6]; break;
-    default: break;
+    case 1: return &d.nsmall[level];
+    case 2: return &d.work[level];
+    case 3: return &d.ntiny[level];
+    case 4: return &d.nmicro[level];
+    case 5: return &d.nmid[level];
+    default: return &d.nrec[3 * level + cls - 6];
   }
-  uint32_t at = 0u;
-  if (count && lane == leader) at = atomicAdd(count, static_cast<uint32_t>(__popc(same)));
-  at = __shfl_sync(0xFFFFFFFFu, at, leader) + __popc(same & ((1u << lane) - 1u));
+}
+
+__device__ __forceinline__ void list_put(const Dev& d, int cls, uint32_t at, uint32_t k) {
   switch (cls) {
     case 1: d.small[at] = k; break;
     case 2: d.big[at] = k; break;
@@ -58,6 +51,29 @@ __device__ __forceinline__ void list_node(const Dev& d, int level, int cls, uint
     case 8: d.rec2[d.rec2_cap - 1u - at] = k; break;
     default: break;
   }
+}
+
+// Appends nodes k and k + 1 to the level's lists of their classes (0: none);
+// all lanes of the warp together, one atomic per class and warp, all classes'
+// at once.  Siblings stay neighbours: their rows share cache lines, and so do
+// the nodes that a warp of the split kernels takes together.
+__device__ __forceinline__ void list_pair(const Dev& d, int level, int cls0, int cls1, uint32_t k) {
+  const int lane = static_cast<int>(threadIdx.x & 31u);
+  const unsigned lt = (1u << lane) - 1u;
+  uint32_t n = 0u, at0 = 0u, at1 = 0u;
+#pragma unroll
+  for (int c = 1; c <= 8; ++c) {
+    const unsigned m0 = __ballot_sync(0xFFFFFFFFu, cls0 == c), m1 = __ballot_sync(0xFFFFFFFFu, cls1 == c);
+    const uint32_t before = static_cast<uint32_t>(__popc(m0 & lt) + __popc(m1 & lt));
+    if (lane == c) n = static_cast<uint32_t>(__popc(m0) + __popc(m1));
+    if (cls0 == c) at0 = before;
+    if (cls1 == c) at1 = before + (cls0 == c ? 1u : 0u);
+  }
+  const uint32_t first = n > 0u ? atomicAdd(list_count(d, level, lane), n) : 0u;
+  at0 += __shfl_sync(0xFFFFFFFFu, first, cls0);
+  at1 += __shfl_sync(0xFFFFFFFFu, first, cls1);
+  list_put(d, cls0, at0, k);
+  list_put(d, cls1, at1, k + 1u);
 }
 
 }  // namespace

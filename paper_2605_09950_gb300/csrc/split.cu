@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(256) k_classify(Dev d, int level) {
       else
         d.nd_split[k] = kLeaf;
     }
-    list_node(d, level, cls, k);
+    list_pair(d, level, cls, 0, k);
   }
 }
 
