@@ -303,6 +303,10 @@ static int session_init(boruta_session* s, const uint8_t* X, int64_t ld, const v
   if ((rc = s->alloc(&d.nd_split, P))) return rc;
   if ((rc = s->alloc(&d.nd_child, P))) return rc;
   if (d.permut && (rc = s->alloc(&d.nd_sc, P))) return rc;
+  if (d.permut && d.permut_form == 0 && use_walks(d)) {
+    if ((rc = s->alloc(&d.wt_tree, n_trees + 1))) return rc;
+    CK(static_cast<cudaError_t>(setup_walks()));
+  }
   if ((rc = s->alloc(&d.nd_delta, P))) return rc;
   if ((rc = s->alloc(&d.nd_lrows, P))) return rc;
   if ((rc = s->alloc(&d.nd_ln, P))) return rc;
@@ -690,7 +694,7 @@ static int enqueue_iteration(boruta_session* s, int t, cudaStream_t st) {
   if (d.permut_form == 1)
     nk += launch_forest_permut(d, s->permut_grid, st);
   else if (d.permut)
-    nk += launch_permut(d, s->permut_grid, s->walk_grid, st);
+    nk += launch_permut(d, s->permut_grid, s->walk_grid, s->sms, st);
   else
     nk += launch_treeimp(d, s->tree_grid, st);
   CK_LAUNCH("importance kernels");

@@ -48,6 +48,7 @@ struct Dev {
   uint32_t* nd_lcnt;             // [cap][C]
   int64_t* nd_lS;
   uint32_t *lvl_off, *lvl_cnt;   // [D + 2]
+  uint2* wt_tree;                // [M + 1] walks.cu: a tree's first packed split node and their number; the total
   uint32_t* work;                // [D + 2] per level: number of nodes in `big`
   uint32_t* chunk;               // [kScanBlocks] per-block split counts
   uint32_t* big;                 // [big_cap] this level's active nodes of more rows than the lists below
@@ -172,7 +173,15 @@ size_t packed_bytes(int variant);
 int launch_gather_live(const Dev& d, cudaStream_t st);
 int launch_children(const Dev& d, int level, uint64_t nodes, cudaStream_t st);
 int launch_treeimp(const Dev& d, int grid, cudaStream_t st);
-int launch_permut(const Dev& d, int grid, int walk_grid, cudaStream_t st);
+int launch_permut(const Dev& d, int grid, int walk_grid, int sms, cudaStream_t st);
+// walks.cu: the walks, with records of ldP bytes (0: too long) in shared memory, on `st`
+// Trees of fewer levels stay in L1 (12 jobs of 500 to 50,000 rows, depth 10:
+// 125.2 ms with k_permut, 127.2 with walks.cu), and few rows do not pay for
+// packing the trees.
+inline bool use_walks(const Dev& d) { return d.N >= 8192 && d.D >= 12; }
+uint32_t walk_nodes(int D, int ldP);
+int setup_walks();
+int launch_walks(const Dev& d, int sms, cudaStream_t st);  // Dev::nd_sc, nd_ln, nd_lrows, nd_lcnt are its scratch
 // Xrow (the row-major copy of Xaug): built once per iteration, after the
 // shadows, for the small-node split and the walks
 int launch_transpose(const Dev& d, int grid, cudaStream_t st);

@@ -15,6 +15,7 @@
 #include <cstdint>
 
 #include "lists.cuh"
+#include "loss.cuh"
 
 #ifndef BORUTA_PERMUT_WALKS
 #define BORUTA_PERMUT_WALKS 8  // re-walks of one OOB row advanced together
@@ -508,65 +509,6 @@ __global__ void k_permut_pi(Dev d) {
     d.piv[i] = perm_apply(P, i);
 }
 
-// loss between the unpermuted leaf q and the permuted leaf q2
-__device__ double loss64(const Dev& d, uint32_t q, uint32_t q2) {
-  const double na = static_cast<double>(d.nd_n[q]), nb = static_cast<double>(d.nd_n[q2]);
-  if (d.kind != 0) {
-    const double ma = static_cast<double>(d.nd_S[q]) / na, mb = static_cast<double>(d.nd_S[q2]) / nb;
-    const double df = (ma - mb) * 0x1p-20;
-    return df * df;
-  }
-  const double eps = d.kl_eps;
-  const double norm = 1.0 + static_cast<double>(d.C) * eps;
-  double kl = 0.0;
-  for (int c = 0; c < d.C; ++c) {
-    const double pa = (static_cast<double>(d.nd_cnt[static_cast<int64_t>(q) * d.C + c]) / na + eps) / norm;
-    const double pb = (static_cast<double>(d.nd_cnt[static_cast<int64_t>(q2) * d.C + c]) / nb + eps) / norm;
-    kl += pa * log(pa / pb);
-  }
-  return kl;
-}
-
-// phi(r) = r log r - r + 1 >= 0, accurate near r = 1 (series in r - 1)
-__device__ __forceinline__ float kl_phi(float r) {
-  const float dl = r - 1.0f;
-  if (fabsf(dl) < 0.25f) {
-    // dl^2 * sum_{n=2..14} (-1)^n dl^(n-2) / (n (n-1)), by Horner
-    constexpr float c[13] = {1.0f / 2,   -1.0f / 6,   1.0f / 12,   -1.0f / 20,  1.0f / 30,
-                             -1.0f / 42, 1.0f / 56,   -1.0f / 72,  1.0f / 90,   -1.0f / 110,
-                             1.0f / 132, -1.0f / 156, 1.0f / 182};
-    float s = c[12];
-#pragma unroll
-    for (int m = 11; m >= 0; --m) s = s * dl + c[m];
-    return s * (dl * dl);
-  }
-  return r * logf(r) - dl;
-}
-
-__device__ float loss32(const Dev& d, uint32_t q, uint32_t q2) {
-  const uint32_t na = d.nd_n[q], nb = d.nd_n[q2];
-  if (d.kind != 0) {
-    // mean difference from exact integers: (S_a n_b - S_b n_a) / (n_a n_b)
-    const __int128 num = static_cast<__int128>(d.nd_S[q]) * nb - static_cast<__int128>(d.nd_S[q2]) * na;
-    const u128 mag = num < 0 ? static_cast<u128>(-num) : static_cast<u128>(num);
-    const uint64_t ml[2] = {static_cast<uint64_t>(mag), static_cast<uint64_t>(mag >> 64)};
-    const uint64_t den = static_cast<uint64_t>(na) * nb;
-    const float df = __fdiv_rn(limbs_to_float(ml, 2, -20), limbs_to_float(&den, 1, 0));
-    return df * df;
-  }
-  const float eps = static_cast<float>(d.kl_eps);
-  const float norm = 1.0f + static_cast<float>(d.C) * eps;
-  float kl = 0.0f;
-  for (int c = 0; c < d.C; ++c) {
-    const float pa = __fdiv_rn(__fdiv_rn(static_cast<float>(d.nd_cnt[static_cast<int64_t>(q) * d.C + c]),
-                                         static_cast<float>(na)) + eps, norm);
-    const float pb = __fdiv_rn(__fdiv_rn(static_cast<float>(d.nd_cnt[static_cast<int64_t>(q2) * d.C + c]),
-                                         static_cast<float>(nb)) + eps, norm);
-    kl += pb * kl_phi(__fdiv_rn(pa, pb));
-  }
-  return kl;
-}
-
 // One thread per (tree, OOB row): walk the row's path; for each distinct
 // feature f on it, re-walk from f's first node with x_f replaced by
 // X[pi(i)][f] (all later f nodes use the swapped value too).  Features off
@@ -579,7 +521,7 @@ __device__ float loss32(const Dev& d, uint32_t q, uint32_t q2) {
 // trees: chunk by chunk through all trees, whose node words L2 holds, so that a
 // row's record is read from DRAM once for all of them (N = 1e5, 500 trees of
 // 7,000 nodes: 24.4 -> 18.9 ms).  Large trees: tree by tree, which keeps one
-// tree's nodes in L1 (N = 1e6, 300 trees of 42,000 nodes: 266 ms against 312).
+// tree's nodes in L1 (N = 1e6, 300 trees of 213,000 nodes: 266 ms against 312).
 // PREC: the precision form (0 = FP64 terms, 1 = FP32 terms), a template
 // argument so that each instantiation holds one loss routine.
 __host__ __device__ inline size_t permut_smem_per_warp(int D) {
@@ -766,16 +708,21 @@ __global__ void k_permut_final(Dev d) {
   }
 }
 
-int launch_permut(const Dev& d, int grid, int walk_grid, cudaStream_t st) {
+int launch_permut(const Dev& d, int grid, int walk_grid, int sms, cudaStream_t st) {
   k_permut_pi<<<(d.N + 255) / 256 < 1024 ? (d.N + 255) / 256 : 1024, 256, 0, st>>>(d);
-  k_pack_nodes<<<grid, 256, 0, st>>>(d);
-  const size_t smem = 4 * permut_smem_per_warp(d.D);
-  if (d.precision == 0)
-    k_permut<0><<<walk_grid, 128, smem, st>>>(d);
-  else
-    k_permut<1><<<walk_grid, 128, smem, st>>>(d);
+  int n = 4;
+  if (use_walks(d) && walk_nodes(d.D, d.ldP) > 0u) {
+    n = 2 + launch_walks(d, sms, st);
+  } else {
+    k_pack_nodes<<<grid, 256, 0, st>>>(d);
+    const size_t smem = 4 * permut_smem_per_warp(d.D);
+    if (d.precision == 0)
+      k_permut<0><<<walk_grid, 128, smem, st>>>(d);
+    else
+      k_permut<1><<<walk_grid, 128, smem, st>>>(d);
+  }
   k_permut_final<<<grid, 256, 0, st>>>(d);
-  return 4;
+  return n;
 }
 
 int launch_transpose(const Dev& d, int grid, cudaStream_t st) {
