@@ -51,23 +51,18 @@ WORKLOADS = {
               "Boruta iterations/sec (binary N=1000, p=50, 100 trees, depth 8, impurity importance)", "treeimp"),
 }
 
-# DRAM bytes (read + write) per launch of the histogram kernel, from the ncu
-# capture named beside it, valid only for the kernel source it was taken on
-# (sha-256 prefix of csrc/split.cu); the line reports null otherwise.
-# DRAM bytes (read + write) of the histogram kernel per tree level, from one
-# ncu capture of a whole iteration (the profile named), valid only while the
-# kernel's and its launch code's sources hash to sources_sha16
-TRAFFIC = {
-    "multiclass_N1000000_p500": {"bytes_per_launch": (582.6e9 + 62.35e9) / 20, "sources_sha16": "0c5bad21bed32dbd",
-                                 "profile": "profiles/k_items_band_multiclass_N1000000_p500.md"},
-}
+# DRAM bytes (read + write) of the larger nodes' split kernels per tree level,
+# from one ncu capture of a whole iteration: workload -> bytes_per_launch,
+# sources_sha16 (valid only while the kernels' and their launch code's sources
+# hash to it), profile.  No capture of the present kernels: the line reports null.
+TRAFFIC = {}
 
 
 def kernel_source_sha16():
     """Hash of the histogram kernel's sources and of the host code that sets
     its launches (a recorded traffic figure holds only for these)."""
     h = hashlib.sha256()
-    for name in ("split.cu", "engine.cuh", "api.cu"):
+    for name in ("split.cu", "record.cu", "column.cu", "planes.cuh", "engine.cuh", "api.cu"):
         with open(os.path.join(ROOT, "paper_2605_09950_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
@@ -481,7 +476,8 @@ def run_gpu(args):
                  "l2_gbs": vps * 17 / 1e9, "ms_per_step": ks["imp_ms"] / args.steps,
                  "l2_bytes_per_visit": "17 B: the two children's split words and child indices (16 B) "
                                        "loaded with the row's bin of the tested feature (1 B)",
-                 "kernels": "k_permut_pi + k_permut + k_permut_final (CUDA events around the stage)"}
+                 "kernels": "k_permut_pi, k_walk_trees and k_walks (or k_pack_nodes and k_permut), k_permut_final "
+                            "(CUDA events around the stage)"}
     line = {
         "metric": metric, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": total_ms / args.steps, "higher_is_better": True,
