@@ -10,6 +10,7 @@
 
 #include "boruta.h"
 #include "engine.cuh"
+#include "sizes.h"
 
 using namespace bgb;
 
@@ -32,13 +33,6 @@ int fail(int code, const char* fmt, ...) {
     cudaError_t e_ = (call);                                                              \
     if (e_ != cudaSuccess) return fail(BORUTA_ECUDA, "%s: %s", #call, cudaGetErrorString(e_)); \
   } while (0)
-
-int64_t shadow_count(int64_t p_live) {
-  int64_t n = p_live;
-  if (n <= 0) return 0;
-  while (n < 5) n *= 2;
-  return n;
-}
 
 int64_t isqrt(int64_t v) {
   int64_t r = static_cast<int64_t>(std::sqrt(static_cast<double>(v)));
@@ -269,8 +263,7 @@ static int session_init(boruta_session* s, const uint8_t* X, int64_t ld, const v
   d.ycls = reg ? nullptr : static_cast<const uint8_t*>(y);
   d.yreg = reg ? static_cast<const int64_t*>(y) : nullptr;
 
-  const int64_t p_aug_max = p + shadow_count(p);
-  const int64_t n_sha_max = shadow_count(p);
+  const int64_t p_aug_max = max_augmented(p);
   // node pool: per tree at most min(2^l, N) nodes at depth l
   uint64_t per_tree = 0;
   for (int l = 0; l <= max_depth; ++l) per_tree += std::min<uint64_t>(1ull << l, static_cast<uint64_t>(N));
@@ -282,7 +275,6 @@ static int session_init(boruta_session* s, const uint8_t* X, int64_t ld, const v
 
   if ((rc = s->alloc(&s->live_d, p))) return rc;
   d.live = s->live_d;
-  (void)n_sha_max;
   if ((rc = s->alloc(&d.Xaug, static_cast<size_t>(p_aug_max) * d.ldN))) return rc;
   const size_t MN = static_cast<size_t>(n_trees) * N;
   if ((rc = s->alloc(&d.bootcnt, MN))) return rc;
