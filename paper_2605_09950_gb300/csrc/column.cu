@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(kFinishThreads) k_col_finish(Dev d, int level)
   using P = ColPack<CM>;
   constexpr int kWarps = kFinishThreads / 32;
   extern __shared__ __align__(16) unsigned char raw[];
-  __shared__ uint32_t hist[P::W * 256];
+  __shared__ __align__(16) uint32_t hist[P::W * 256];  // read and cleared 16 bytes at a time
   __shared__ uint32_t red[kWarps], cps[CM], s_sp, s_total;
   uint32_t* bits = reinterpret_cast<uint32_t*>(raw);  // per 32 rows: which go left
   uint32_t* before = bits + (d.N + 31) / 32;          // and how many before them

@@ -400,7 +400,8 @@ __device__ uint32_t warp_partition(const Dev& d, int64_t base, uint32_t len, uin
 // Bins of a lane in histograms of one 32-bit plane of 256 words per field.
 __device__ __forceinline__ int lane_bins(int B) { return B > 128 ? 8 : (B > 64 ? 4 : (B > 32 ? 2 : 1)); }
 
-// A lane's bpl (1, 2, 4 or 8) consecutive bins of a plane.
+// A lane's bpl (1, 2, 4 or 8) consecutive bins of a plane, by 4, 8 or 16 bytes:
+// the plane starts on a 16-byte boundary (p = plane + lane * bpl).
 __device__ __forceinline__ void ld_bins(const uint32_t* p, int bpl, uint32_t (&h)[8]) {
 #pragma unroll
   for (int q = 0; q < 8; ++q) h[q] = 0u;
