@@ -1087,7 +1087,9 @@ int boruta_session_dump(boruta_session* s, int what, void* host, int64_t capacit
       std::vector<uint32_t> off(d.D + 2), cnt(d.D + 2);
       CK(cudaMemcpy(off.data(), d.lvl_off, (d.D + 2) * 4, cudaMemcpyDeviceToHost));
       CK(cudaMemcpy(cnt.data(), d.lvl_cnt, (d.D + 2) * 4, cudaMemcpyDeviceToHost));
-      const uint32_t total = off[d.D] + cnt[d.D];
+      const uint32_t total = off[d.D] + cnt[d.D];  // places of the pool: a level starts at an even one
+      int64_t nodes = 0;
+      for (int l = 0; l <= d.D; ++l) nodes += cnt[l];
       std::vector<uint32_t> tree(total), heap(total), len(total), n(total), split(total);
       std::vector<double> delta(total);
       std::vector<uint32_t> cnts(d.kind ? 0 : static_cast<size_t>(total) * d.C);
@@ -1131,7 +1133,7 @@ int boruta_session_dump(boruta_session* s, int what, void* host, int64_t capacit
         for (int tau = 0; tau < d.M; ++tau) o[tau + 1] = o[tau] + static_cast<int64_t>(per[tau].size());
         return 0;
       }
-      const int64_t need = static_cast<int64_t>(total) * sizeof(boruta_node);
+      const int64_t need = nodes * static_cast<int64_t>(sizeof(boruta_node));
       if (bytes) *bytes = need;
       if (!host) return 0;
       if (capacity < need) return fail(BORUTA_EINVAL, "capacity too small");
