@@ -15,7 +15,7 @@ CSRC = os.path.join(PKG, "csrc")
 OUT_DIR = os.path.join(PKG, "_build")
 LIB = os.path.join(OUT_DIR, "libboruta_gb300.so")
 SOURCES = ["api.cu", "kernels.cu", "split.cu", "small.cu", "record.cu", "threebin.cu", "regress.cu", "column.cu", "walks.cu", "noalloc.cu", "quantise.cu", "rank.cu"]
-HEADERS = ["device.cuh", "engine.cuh", "split.cuh", "regress.cuh", "planes.cuh", "lists.cuh", "loss.cuh", "sizes.h"]
+HEADERS = ["device.cuh", "engine.cuh", "split.cuh", "regress.cuh", "planes.cuh", "lists.cuh", "loss.cuh", "sizes.h", "routes.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # -fmad=false: no multiply-add contraction, so every floating-point operation
 # of the exact-rounding contract is rounded on its own (matches the CPU oracle).

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "device.cuh"
+#include "routes.h"
 
 namespace bgb {
 
@@ -175,10 +176,7 @@ int launch_children(const Dev& d, int level, uint64_t nodes, cudaStream_t st);
 int launch_treeimp(const Dev& d, int grid, cudaStream_t st);
 int launch_permut(const Dev& d, int grid, int walk_grid, int sms, cudaStream_t st);
 // walks.cu: the walks, with records of ldP bytes (0: too long) in shared memory, on `st`
-// Trees of fewer levels stay in L1 (12 jobs of 500 to 50,000 rows, depth 10:
-// 125.2 ms with k_permut, 127.2 with walks.cu), and few rows do not pay for
-// packing the trees.
-inline bool use_walks(const Dev& d) { return d.N >= 8192 && d.D >= 12; }
+inline bool use_walks(const Dev& d) { return walks_pay(d.kind == 0, d.precision != 0, d.N, d.M, d.D); }
 uint32_t walk_nodes(int D, int ldP);
 int setup_walks();
 int launch_walks(const Dev& d, int sms, cudaStream_t st);  // Dev::nd_sc, nd_ln, nd_lrows, nd_lcnt are its scratch

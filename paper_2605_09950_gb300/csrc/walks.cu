@@ -10,8 +10,8 @@
 // levels of the largest trees are still read from L2.
 //
 //   k_walk_trees  a block per tree: numbers its split nodes in level order and
-//                 writes them packed; for FP32 terms also each leaf's class
-//                 probabilities, divided once per leaf.
+//                 writes them packed; for classes (FP32 terms) also each
+//                 leaf's probabilities, divided once per leaf.
 //   k_walks       blocks take 2048 rows of a tree at a time, a warp 3 rows: a
 //                 lane per row walks the path; then a lane per path node finds
 //                 the re-walks (ballots and matches over the path's features);
@@ -22,7 +22,7 @@
 // Measured: N = 1e6, p = 500, 300 trees, depth 20 (213,000 nodes a tree): 963 ->
 // 889 ms an iteration; N = 1e5, p = 1000, 500 trees, depth 16: 86.4 -> 80.0.
 // Bound by issue (about 750 warp instructions a row and tree, a third of them
-// the losses) and by the latency of a step.
+// the losses) and by the latency of a step.  Which forests it takes: routes.h.
 #include <algorithm>
 #include <cstdint>
 
@@ -152,6 +152,7 @@ __device__ __forceinline__ float loss_probs(const Dev& d, uint32_t q, uint32_t q
   return kl;
 }
 
+// PREC: the terms' precision (0, FP64: regression only; walks_pay in routes.h)
 template <int PREC>
 __global__ void __launch_bounds__(kWarps * 32, 1) k_walks(Dev d, uint32_t nodes) {
   extern __shared__ __align__(16) unsigned char smem[];
