@@ -21,7 +21,8 @@
 //   value's own bucket, if any.  Where too many keys fall into the targets'
 //   buckets (heavily repeated values), a sweep finds the buckets that hold one
 //   distinct key, whose targets are that key; if that does not thin them out
-//   either, all targets are found by bisection over the column, 32 sweeps.
+//   either, all targets are found by bisection over the column, from their
+//   buckets' least and greatest keys.
 // Bound by the three reads (13 bytes a value moved against 5) and the shared
 // atomics.  Measured at N = 1e6, p = 500, B = 256: 3.0 ms (32 sweeps with
 // a binary search per value before: 81.9 ms); N = 1000, p = 50, B = 64, the
@@ -101,23 +102,26 @@ __device__ __forceinline__ bool sweep(const float* col, uint32_t N, F&& f) {
   return nan;
 }
 
-// All targets by bisection on the key, one sweep per key bit: every target
-// keeps an interval [lo_k, hi_k]; the intervals stay ordered in k (the targets
-// are), so the midpoints are sorted and one sweep counts for every midpoint
-// the values at or below it.  Result in lo.
+// All targets by bisection on the key, one sweep per halving: every target
+// keeps an interval [lo_k, hi_k], at first the least and the greatest key of
+// its bucket; the intervals stay ordered in k (the targets are), so the
+// midpoints are sorted and one sweep counts for every midpoint the values at
+// or below it.  A bucket spans at most 20 bits of the key, and 20 - m where it
+// holds many of the values (2^m at least its cell's sample count), so columns of
+// close repeated values, which come here, take few sweeps (200 neighbouring
+// floats, 1000 columns, B = 64: N = 20000 1.35 ms, 1e5 3.8 ms; from the whole key
+// range, 33 sweeps, 3.9 and 12.0 ms).  Result in lo.
 __device__ void bisect_column(const float* col, uint32_t N, int B, uint32_t* lo, uint32_t* hi, uint32_t* mid,
                               uint32_t* cnt) {
   const int nt = B - 1;
-  for (int k = threadIdx.x; k < nt; k += blockDim.x) {
-    lo[k] = 0u;
-    hi[k] = 0xFFFFFFFFu;
-  }
-  __syncthreads();
-  for (int pass = 0; pass < 33; ++pass) {
-    for (int k = threadIdx.x; k < nt; k += blockDim.x)
+  for (int pass = 0; pass < 33; ++pass) {  // (an open interval halves: at most 32)
+    int open = 0;
+    for (int k = threadIdx.x; k < nt; k += blockDim.x) {
+      open |= lo[k] < hi[k];
       mid[k] = static_cast<uint32_t>((static_cast<uint64_t>(lo[k]) + hi[k]) >> 1);
+    }
     for (int k = threadIdx.x; k <= nt; k += blockDim.x) cnt[k] = 0u;
-    __syncthreads();
+    if (!__syncthreads_or(open)) break;
     // cnt[c] = values whose key lies above exactly c midpoints
     sweep(col, N, [&](uint32_t, uint32_t key) { atomicAdd(&cnt[count_below(mid, nt, key)], 1u); });
     __syncthreads();
@@ -374,7 +378,12 @@ __global__ void __launch_bounds__(kQThreads, 2) k_quantise(const float* X, int64
         if (lane == 0u) sm.T[k] = lo;
       }
     } else {
-      bisect_column(col, N, B, sm.T, sm.mx, sm.cur, sm.start);
+      for (int k = tid; k < nt; k += kQThreads) {
+        sm.T[k] = sm.mn[sm.head[k]];
+        sm.size[k] = sm.mx[sm.head[k]];
+      }
+      __syncthreads();
+      bisect_column(col, N, B, sm.T, sm.size, sm.cur, sm.start);
     }
     __syncthreads();
     // ---- sweep 3: bin = number of targets below the value
