@@ -527,23 +527,25 @@ int boruta_session_create(const uint8_t* X, int64_t ld, const void* y, int64_t N
 // classes) records win at every size the tiles hold (10.2 -> 8.1 ms an
 // iteration); from DRAM the two cross at about N / 64 rows (N = 1e5, p = 1000:
 // 146.6 ms at N / 64, 151 at N / 32, 157 at N / 8, 164 without; N = 1e6: 955
-// against 1148 ms without, the same from N / 64 to N / 256).  Columns of at
-// most 4 bins stay with the register counts of the column path.
+// against 1148 ms without, the same from N / 64 to N / 256).  With few sampled
+// columns or trees they do not pay (records_pay).  Columns of at most 4 bins stay
+// with the register counts of the column path.
 static uint32_t record_rows(const boruta_session* s, const Dev& d) {
-  if (d.kind != 0 || s->split_path != 0 || d.B <= 4) return 0u;
+  if (d.kind != 0 || s->split_path != 0 || d.B <= 4 || !records_pay(d.N, d.M, d.mtry)) return 0u;
   const bool in_l2 = static_cast<uint64_t>(d.N) * static_cast<uint64_t>(d.ldP) <= (96ull << 20);
   return std::min<uint32_t>(kRecordRows, static_cast<uint32_t>(d.N) / (in_l2 ? 1u : 64u));
 }
 
 // Whether column.cu takes the classification nodes of more than 256 rows: the
-// columns fit in shared memory (N up to about 130,000 to 200,000, by classes).
+// columns fit in shared memory (N up to about 130,000 to 200,000, by classes),
+// and there is enough for it to do (columns_pay).
 // Measured against record.cu and the band path (ms an iteration): N = 5003, 3
 // classes 3.34 -> 3.09; N = 30011, 8 classes 8.05 -> 6.79; N = 1e5, p = 1000
 // 141 -> 93; 12 jobs of 500 to 50,000 rows 165 -> 137.  Up to 4096 rows
 // record.cu holds every node in one launch.
 static int32_t use_columns(const boruta_session* s, const Dev& d) {
   if (d.kind != 0 || s->split_path != 0 || s->col_grid == 0 || d.B <= 4) return 0;
-  if (d.N <= static_cast<int32_t>(kRecordRows)) return 0;
+  if (d.N <= static_cast<int32_t>(kRecordRows) || !columns_pay(d.N, d.M, d.mtry)) return 0;
   const uint64_t nodes = static_cast<uint64_t>(d.M) * (static_cast<uint64_t>(d.N) / 257 + 1);
   return nodes * static_cast<uint64_t>(d.mtry) <= d.item_cap;
 }

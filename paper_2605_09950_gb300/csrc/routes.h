@@ -29,4 +29,34 @@ inline bool walks_pay(bool classification, bool fp32, int64_t N, int64_t trees, 
   return fp32 && rows >= (depth < 20 ? 5000000 : 2000000);
 }
 
+// Classification nodes above 64 rows in problems of 65,536 rows and more, whose
+// nodes of weight 65,536 and up are counted by column gathers in feature bands
+// in any case.  column.cu and record.cu then run before the band kernels of
+// every level, and the longest node of each is waited for in turn; with few
+// (node, column) items, which leave the GPU idle, the bands alone take all the
+// nodes of a level together in less time.  Both lines by the columns a node
+// samples and the trees; below 65,536 rows (and a little above, where few
+// levels hold both) there is no second wait, and the rules say yes.
+// Split stage, bands alone -> column.cu, ms (2 / 5 classes, depth 12):
+//   N = 60000, 30 trees, 10 columns    3.8 -> 2.9 (5)
+//   N = 80000, 60 trees, 4 / 10 / 31   1.04, 0.91 / 1.11, 0.93 / 1.20, 1.17 times
+//   N = 1e5, 1 tree, any sample        1.1 to 1.5 times as fast
+//   N = 1e5, 30 trees, 10 / 31 / 63    0.97, 0.91 / 0.95, 0.89 / 1.24, 1.10 times
+//   N = 1e5, 200 trees, 4 / 20 / 44    0.85, 0.80 / 1.03, 1.05 / 1.37, 1.22 times
+//   N = 130000, 60 trees, 10 / 31 / 63 0.82, 0.78 / 0.92, 0.86 / 1.22, 1.13 times
+inline bool columns_pay(int64_t N, int64_t trees, int64_t mtry) {
+  if (N < (mtry >= 8 ? 81920 : 72000) || mtry >= 44 || trees <= 3) return true;
+  return 14 * trees * mtry >= N - 65536;
+}
+
+// Bands alone -> record.cu (where column.cu does not take the problem), times as
+// fast, 5 classes:
+//   N = 2e5, depth 12, 100 trees, 4 / 10 / 31 / 63 columns  0.87 / 0.89 / 1.07 / 1.24
+//   N = 2e5, depth 12, 10 trees                             0.87 / 0.86 / 0.92 / 1.07
+//   N = 2e5, depth 20, 100 trees                            0.78 / 0.89 / 1.18 / 1.35
+//   N = 1e6, depth 20, 300 trees, 10 / 31 columns           0.87 / 1.15
+inline bool records_pay(int64_t N, int64_t trees, int64_t mtry) {
+  return N < 65536 || mtry >= 48 || (mtry >= 24 && trees * mtry >= 900);
+}
+
 }  // namespace bgb

@@ -38,3 +38,19 @@ WALKS = [("walks_pay(true, true, 1000000, 300, 20)", 1), ("walks_pay(true, true,
 
 def test_walks(tmp_path):
     check(tmp_path, WALKS)
+
+
+# columns_pay(N, trees, mtry), records_pay(N, trees, mtry)
+LARGE_CLASSIFICATION = [
+    ("columns_pay(30011, 100, 20)", 1), ("columns_pay(65535, 1, 1)", 1), ("columns_pay(66000, 200, 4)", 1),
+    ("columns_pay(80000, 200, 4)", 0), ("columns_pay(80000, 60, 31)", 1),
+    ("columns_pay(100000, 500, 44)", 1), ("columns_pay(100000, 200, 31)", 1), ("columns_pay(100000, 1, 4)", 1),
+    ("columns_pay(100000, 30, 31)", 0), ("columns_pay(100000, 100, 10)", 0), ("columns_pay(100000, 200, 4)", 0),
+    ("columns_pay(130000, 60, 31)", 0), ("columns_pay(130000, 200, 10)", 0), ("columns_pay(130000, 200, 44)", 1),
+    ("records_pay(4000, 1, 1)", 1), ("records_pay(1000000, 300, 31)", 1), ("records_pay(200000, 100, 31)", 1),
+    ("records_pay(200000, 10, 63)", 1), ("records_pay(200000, 100, 10)", 0), ("records_pay(400000, 300, 10)", 0),
+    ("records_pay(1000000, 10, 14)", 0), ("records_pay(400000, 10, 20)", 0)]
+
+
+def test_large_classification(tmp_path):
+    check(tmp_path, LARGE_CLASSIFICATION)
