@@ -579,7 +579,9 @@ static int enqueue_iteration(boruta_session* s, int t, cudaStream_t st) {
                  8ll * d.mtry >= p_aug;
   // regress.cu: columns of more than 4 bins (fewer are counted in registers by
   // the column path), lists of 16-bit columns
-  if (d.kind == 1 && d.B > 4 && s->split_path == 0 && d.mtry <= kRegColumns && p_aug <= 65536)
+  const bool reg_ok = d.kind == 1 && d.B > 4 && s->split_path == 0 && d.mtry <= kRegColumns && p_aug <= 65536;
+  d.reg_rows = reg_ok && reg_rows_pays(d.N, d.mtry);
+  if (reg_ok && reg_record_pays(d.N, d.M, d.mtry))
     d.rec_rows = std::min<uint32_t>(kRegRecordRows, static_cast<uint32_t>(d.N));
   // feature bands: ~kBandBytes of columns each, at most kMaxBands; the packed
   // item holds a 14-bit slot and a 22-bit feature

@@ -68,6 +68,7 @@ struct Dev {
   uint32_t rec_rows;             // largest node split by record (0: none)
   int32_t columns;               // 1: classification nodes of more than 256 rows, weight below 65536, go to
                                  //   column.cu (listed in rec2 from its start), rec_rows = 256
+  int32_t reg_rows;              // 1: regression nodes of at most 32 rows go to regress.cu (else k_split_small)
   uint32_t* col_cnt;             // [p_aug] items per column, then their ends
   int32_t wide_y;                // regression: a row's weighted target may exceed 41 bits and its sign, or a
                                  //   sum of them 2^53
@@ -156,8 +157,8 @@ int launch_record(const Dev& d, int level, const int* grids, uint64_t nodes, cud
 // nodes below kThreeRows rows, the smallest on `st2`
 int setup_three_bins(int p_aug, int sms, int* grids);
 int launch_three_bins(const Dev& d, int level, const int* grids, uint64_t nodes, cudaStream_t st, cudaStream_t st2);
-// regress.cu: grid sizes; the level's regression nodes of at most rec_rows
-// rows (d.rec_rows > 0), those of at most 32 on `st2`
+// regress.cu: grid sizes; the level's regression nodes of 33 to rec_rows rows
+// (none where d.rec_rows is 0), and on `st2` those of at most 32 if d.reg_rows
 int setup_regress(int sms, int* grids);
 int launch_regress(const Dev& d, int level, const int* grids, uint64_t nodes, cudaStream_t st, cudaStream_t st2);
 // column.cu: whether it can take the session's columns (grid of its last

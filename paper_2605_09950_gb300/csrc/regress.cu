@@ -521,13 +521,19 @@ int launch_regress(const Dev& d, int level, const int* grids, uint64_t nodes, cu
     return static_cast<unsigned>(std::max<uint64_t>(1, std::min<uint64_t>(static_cast<uint64_t>(grids[i]), most)));
   };
   const uint64_t M = static_cast<uint64_t>(d.M), N = static_cast<uint64_t>(d.N);
-  k_reg_rows<<<grid(2, (nodes + 7) / 8), 256, 0, st2>>>(d, level);
-  int n = 2;
+  int n = 0;
+  if (d.reg_rows) {
+    k_reg_rows<<<grid(2, (nodes + 7) / 8), 256, 0, st2>>>(d, level);
+    ++n;
+  }
   if (d.rec_rows > 256u) {
     k_reg_record<1024, 8, 2><<<grid(1, std::min(nodes, M * (N / 257 + 1))), 256, sizeof(RegSmem<1024, 8>), st>>>(d, level);
     ++n;
   }
-  k_reg_record<256, 4, 5><<<grid(0, std::min(nodes, M * (N / 33 + 1))), 128, sizeof(RegSmem<256, 4>), st>>>(d, level);
+  if (d.rec_rows > 0u) {
+    k_reg_record<256, 4, 5><<<grid(0, std::min(nodes, M * (N / 33 + 1))), 128, sizeof(RegSmem<256, 4>), st>>>(d, level);
+    ++n;
+  }
   return n;
 }
 

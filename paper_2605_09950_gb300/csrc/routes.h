@@ -37,20 +37,21 @@ inline bool walks_pay(bool classification, bool fp32, int64_t N, int64_t trees, 
 // nodes of a level together in less time.  Both lines by the columns a node
 // samples and the trees; below 65,536 rows (and a little above, where few
 // levels hold both) there is no second wait, and the rules say yes.
-// Split stage, bands alone -> column.cu, ms (2 / 5 classes, depth 12):
-//   N = 60000, 30 trees, 10 columns    3.8 -> 2.9 (5)
-//   N = 80000, 60 trees, 4 / 10 / 31   1.04, 0.91 / 1.11, 0.93 / 1.20, 1.17 times
-//   N = 1e5, 1 tree, any sample        1.1 to 1.5 times as fast
-//   N = 1e5, 30 trees, 10 / 31 / 63    0.97, 0.91 / 0.95, 0.89 / 1.24, 1.10 times
-//   N = 1e5, 200 trees, 4 / 20 / 44    0.85, 0.80 / 1.03, 1.05 / 1.37, 1.22 times
-//   N = 130000, 60 trees, 10 / 31 / 63 0.82, 0.78 / 0.92, 0.86 / 1.22, 1.13 times
+// Split stage, column.cu against the bands alone, times as fast (2, 5 classes,
+// depth 12):
+//   N = 60000, 30 trees, 10 / 31 columns      2.20, 1.49 / 1.95, 1.61
+//   N = 80000, 60 trees, 4 / 10 / 31          1.04, 0.91 / 1.11, 0.93 / 1.20, 1.17
+//   N = 1e5, 1 tree, 4 / 63                   1.12, 1.14 / 1.50, 1.48
+//   N = 1e5, 30 trees, 10 / 31 / 63           0.97, 0.91 / 0.95, 0.89 / 1.24, 1.10
+//   N = 1e5, 200 trees, 4 / 20 / 44           0.85, 0.80 / 1.03, 1.05 / 1.37, 1.22
+//   N = 130000, 60 trees, 10 / 31 / 63        0.82, 0.78 / 0.92, 0.86 / 1.22, 1.13
 inline bool columns_pay(int64_t N, int64_t trees, int64_t mtry) {
   if (N < (mtry >= 8 ? 81920 : 72000) || mtry >= 44 || trees <= 3) return true;
   return 14 * trees * mtry >= N - 65536;
 }
 
-// Bands alone -> record.cu (where column.cu does not take the problem), times as
-// fast, 5 classes:
+// record.cu (where column.cu does not take the problem) against the bands alone,
+// times as fast, 5 classes:
 //   N = 2e5, depth 12, 100 trees, 4 / 10 / 31 / 63 columns  0.87 / 0.89 / 1.07 / 1.24
 //   N = 2e5, depth 12, 10 trees                             0.87 / 0.86 / 0.92 / 1.07
 //   N = 2e5, depth 20, 100 trees                            0.78 / 0.89 / 1.18 / 1.35
@@ -58,5 +59,27 @@ inline bool columns_pay(int64_t N, int64_t trees, int64_t mtry) {
 inline bool records_pay(int64_t N, int64_t trees, int64_t mtry) {
   return N < 65536 || mtry >= 48 || (mtry >= 24 && trees * mtry >= 900);
 }
+
+// Regression over more than 4 bins.  Nodes of 33..1024 rows by regress.cu's
+// blocks (else the column gathers): a block reads 32 columns of its node at a
+// time and deals them to its warps, so few sampled columns leave it idle; up to
+// 1024 rows the gathers' launches go too.  Split stage, k_reg_record against the
+// gathers, times as fast (depth 12, 1 / 10 / 100 trees):
+//   N = 1000, 4 / 33 columns      1.99 / 1.64 / 1.46    3.17 / 2.47 / 1.84
+//   N = 2000, 10 / 16 / 24        1.21 / 1.01 / 0.86    1.47 / 1.14 / 1.01    1.67 / 1.19 / 1.08
+//   N = 5000, 33 / 48 / 64        1.33 / 1.04 / 0.79    1.46 / 1.17 / 0.90    1.83 / 1.36 / 0.99
+//   N = 20000, 33 / 64 / 133      1.13 / 0.88 / 0.83    1.20 / 1.08 / 1.08    1.48 / 1.27 / 1.29
+//   N = 1e5, 33 / 64 / 133        0.92 / 0.89 / 0.91    0.99 / 1.05 / 1.05    1.10 / 1.22 / 1.18
+inline bool reg_record_pays(int64_t N, int64_t trees, int64_t mtry) {
+  if (N <= 1024 || mtry >= 64 || N <= 128 * mtry) return true;
+  return (mtry >= 24 && N * trees <= 50000) || (mtry >= 48 && N * trees <= 200000);
+}
+
+// Nodes of at most 32 rows by its warps (else k_split_small): their products take
+// 32 columns at a time.  Split stage, times as fast (depth 16, 100 trees, 4 / 16 /
+// 24 / 48 columns): N = 2000 0.99 / 1.11 / 1.20 / 1.50, N = 5000 0.87 / 0.97 / 1.09 /
+// 1.32, N = 20000 0.85 / 0.93 / 1.00 / 1.14, N = 1e5 0.94 / 0.97 / 1.01 / 1.05; 10
+// trees 0.99 to 1.05 below 24 columns, more above.
+inline bool reg_rows_pays(int64_t N, int64_t mtry) { return N <= 2048 || mtry >= 24; }
 
 }  // namespace bgb

@@ -312,7 +312,8 @@ __device__ void small_node(const Dev& d, int level, uint32_t k, uint8_t* sbin, u
 // SEG = 8: one warp per four micro nodes (a quarter warp each); SEG = 16:
 // one warp per pair of tiny nodes (a half warp each); SEG = 32: one warp per
 // small node.  Regression nodes that regress.cu and threebin.cu do not take
-// (more than kRegColumns sampled columns, four bins, split_path = 1).
+// (more than kRegColumns sampled columns, few of them (reg_rows_pays), at most
+// four bins, split_path = 1).
 template <int SEG>
 __global__ void __launch_bounds__(256, BORUTA_SMALL_MINB) k_split_small(Dev d, int level) {
   __shared__ uint8_t sbins[8][kSmallAhead * 32];
@@ -1501,13 +1502,14 @@ int launch_level(const Dev& d, int level, int grid_small, int grid_items, const 
     if (d.columns) n += launch_column(d, level, sms, grid_rec[1], std::min(nodes, static_cast<uint64_t>(d.rec2_cap)), st);
   } else if (d.three_bins) {
     n += launch_three_bins(d, level, grid_rec, nodes, st, st2);
-  } else if (d.rec_rows > 0u) {
-    n += launch_regress(d, level, grid_rec, nodes, st, st2);
   } else {
-    k_split_small<8><<<grid_small, 256, 0, st2>>>(d, level);
-    k_split_small<16><<<grid_small, 256, 0, st2>>>(d, level);
-    k_split_small<32><<<grid_small, 256, 0, st2>>>(d, level);
-    n += 3;
+    if (!d.reg_rows) {
+      k_split_small<8><<<grid_small, 256, 0, st2>>>(d, level);
+      k_split_small<16><<<grid_small, 256, 0, st2>>>(d, level);
+      k_split_small<32><<<grid_small, 256, 0, st2>>>(d, level);
+      n += 3;
+    }
+    n += launch_regress(d, level, grid_rec, nodes, st, st2);
   }
   cudaEventRecord(join, st2);
   if (static_cast<uint32_t>(d.N) <= taken) {  // no node is larger

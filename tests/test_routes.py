@@ -54,3 +54,18 @@ LARGE_CLASSIFICATION = [
 
 def test_large_classification(tmp_path):
     check(tmp_path, LARGE_CLASSIFICATION)
+
+
+# reg_record_pays(N, trees, mtry), reg_rows_pays(N, mtry)
+REGRESSION = [("reg_record_pays(1000, 100, 1)", 1), ("reg_record_pays(2000, 100, 24)", 1),
+              ("reg_record_pays(10000, 100, 100)", 1), ("reg_record_pays(100000, 10, 133)", 1),
+              ("reg_record_pays(5000, 1, 33)", 1), ("reg_record_pays(5000, 10, 48)", 1),
+              ("reg_record_pays(2000, 100, 10)", 0), ("reg_record_pays(5000, 100, 33)", 0),
+              ("reg_record_pays(20000, 10, 33)", 0), ("reg_record_pays(20000, 100, 33)", 0),
+              ("reg_record_pays(100000, 100, 33)", 0),
+              ("reg_rows_pays(1000, 1)", 1), ("reg_rows_pays(2000, 4)", 1), ("reg_rows_pays(20000, 33)", 1),
+              ("reg_rows_pays(100000, 133)", 1), ("reg_rows_pays(20000, 10)", 0), ("reg_rows_pays(5000, 4)", 0)]
+
+
+def test_regression(tmp_path):
+    check(tmp_path, REGRESSION)
