@@ -82,4 +82,26 @@ inline bool reg_record_pays(int64_t N, int64_t trees, int64_t mtry) {
 // trees 0.99 to 1.05 below 24 columns, more above.
 inline bool reg_rows_pays(int64_t N, int64_t mtry) { return N <= 2048 || mtry >= 24; }
 
+// Regression over at most 3 bins by threebin.cu (else by row, and the column
+// gathers' register counts).  Its blocks read records whole, 1024 columns a
+// round, and score the sampled ones: worth it while a node samples many of them,
+// or while there is so little to do that the launches count.  Split stage, times
+// as fast (depth 10):
+//   N = 1000, 100 trees, 6 / 24 / 48 columns    1.16 / 2.00 / 3.09 (p = 24)
+//   N = 2000, 100 trees, 16 / 40                1.13 / 1.64 (p = 24, 60; iteration)
+//   N = 2000, 300 trees, 16 / 40                0.73 / 1.19 (p = 24, 60; iteration)
+//   N = 5000, 10 trees, 6 / 24 / 48             1.17 / 1.81 / 2.59 (p = 24)
+//   N = 5000, 100 trees, 6 / 24 / 48            0.49 / 0.86 / 1.30 (p = 24)
+//   N = 5000, 100 trees, 50 / 100 / 400         1.19 / 2.06 / 5.82 (p = 200)
+//   N = 16000, 100 trees, 13 / 50 / 100         0.45 / 0.99 / 1.82 (p = 50)
+//   N = 40000, 10 trees, 13 / 50 / 100          0.61 / 0.84 / 1.33 (p = 50)
+//   N = 30000, 100 trees, 40 / 66               0.85 / 1.22 (p = 60, 100; iteration)
+//   N = 40000, 1 tree, 500 / 1000 of 4000       0.66 / 1.21
+// From 16,384 rows on the largest nodes go to the gathers in any case.
+inline bool three_bins_pay(int64_t N, int64_t trees, int64_t mtry, int64_t columns) {
+  if (8 * mtry < columns || (N >= 16384 && 4 * mtry < columns)) return false;
+  if (mtry >= 64 || (mtry >= 40 && N <= 5000) || (mtry >= 24 && N <= 1024)) return true;
+  return N <= 5000 && N * trees <= (mtry >= 16 ? 200000 : 100000);
+}
+
 }  // namespace bgb

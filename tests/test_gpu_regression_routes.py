@@ -1,7 +1,8 @@
 """Regression over more than 4 bins, at the sizes where a node's kernel changes
 with the rows and the sampled columns (reg_record_pays, reg_rows_pays): nodes of
 33 to 1024 rows by blocks or by the column gathers, nodes of at most 32 rows by
-matrix products or by row; every tree against the CPU oracle, bit for bit."""
+matrix products or by row; genotype columns on both sides of three_bins_pay;
+every tree against the CPU oracle, bit for bit."""
 import numpy as np
 import pytest
 
@@ -24,3 +25,16 @@ def test_regression_routes(N, mtry, bins, depth, tie_break):
     y = X[0, :N].astype(np.int64) * 2**17 - X[7, :N].astype(np.int64) * 2**16 + rng.integers(-2**21, 2**21, N)
     w = synth.Workload("t", X, y, N, p, synth.REGRESSION | synth.TREEIMP, 1, bins, 4, depth, 2, seed=N, mtry=mtry)
     check_iteration(w, tie_break=tie_break)
+
+
+@pytest.mark.parametrize("tie_break", [0, 1])
+@pytest.mark.parametrize("N,p,bins,n_trees,depth", [
+    (2500, 20, 3, 40, 9), (2500, 20, 3, 41, 9), (17_001, 60, 3, 4, 6),  # records; by row (13 and 40 columns)
+    (16_400, 150, 3, 2, 5), (27_000, 150, 2, 2, 3)])  # records, and nodes of more than 16383 rows by column
+def test_three_bin_routes(N, p, bins, n_trees, depth, tie_break):
+    rng = np.random.default_rng(N + p)
+    X = np.zeros((p, synth.pad16(N)), np.uint8)
+    X[:, :N] = rng.integers(0, bins, size=(p, N))
+    y = X[0, :N].astype(np.int64) * 2**20 - X[7, :N].astype(np.int64) * 2**19 + rng.integers(-2**21, 2**21, N)
+    w = synth.Workload("t", X, y, N, p, synth.REGRESSION | synth.TREEIMP, 1, bins, n_trees, depth, 2, seed=N, mtry=0)
+    check_iteration(w, trees=[0, n_trees - 1], tie_break=tie_break)

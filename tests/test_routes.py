@@ -69,3 +69,18 @@ REGRESSION = [("reg_record_pays(1000, 100, 1)", 1), ("reg_record_pays(2000, 100,
 
 def test_regression(tmp_path):
     check(tmp_path, REGRESSION)
+
+
+# three_bins_pay(N, trees, mtry, columns)
+THREE_BINS = [("three_bins_pay(20000, 100, 3335, 10006)", 1), ("three_bins_pay(1000, 100, 6, 48)", 1),
+              ("three_bins_pay(5000, 10, 6, 48)", 1), ("three_bins_pay(5000, 100, 133, 400)", 1),
+              ("three_bins_pay(16000, 100, 100, 100)", 1), ("three_bins_pay(40000, 100, 100, 400)", 1),
+              ("three_bins_pay(2000, 100, 16, 48)", 1), ("three_bins_pay(2000, 300, 40, 120)", 1),
+              ("three_bins_pay(30000, 100, 66, 200)", 1), ("three_bins_pay(2000, 300, 16, 48)", 0),
+              ("three_bins_pay(5000, 100, 24, 48)", 0), ("three_bins_pay(16000, 100, 33, 100)", 0),
+              ("three_bins_pay(40000, 10, 33, 100)", 0), ("three_bins_pay(40000, 1, 500, 4000)", 0),
+              ("three_bins_pay(300, 10, 10, 100)", 0)]
+
+
+def test_three_bins(tmp_path):
+    check(tmp_path, THREE_BINS)
