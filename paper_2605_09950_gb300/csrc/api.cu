@@ -682,7 +682,8 @@ static int enqueue_iteration(boruta_session* s, int t, cudaStream_t st) {
                        timed ? s->hev[2 * level] : nullptr, timed ? s->hev[2 * level + 1] : nullptr);
     CK_LAUNCH("split kernels");
     if (timed) CK(cudaEventRecord(s->ev[2 * level + 1], st));
-    nk += launch_children(d, level, nodes, st);
+    nk += launch_children(d, level, nodes, static_cast<uint64_t>(d.M) * std::min<uint64_t>(2 * width, static_cast<uint64_t>(d.N)),
+                          st);
     CK_LAUNCH("next-level kernels");
   }
   if (timed) CK(cudaEventRecord(s->iev[0], st));

@@ -173,7 +173,7 @@ const void* small_kernel_ptr(int variant);  // for its occupancy
 size_t cand_bytes(int variant);
 size_t packed_bytes(int variant);
 int launch_gather_live(const Dev& d, cudaStream_t st);
-int launch_children(const Dev& d, int level, uint64_t nodes, cudaStream_t st);
+int launch_children(const Dev& d, int level, uint64_t nodes, uint64_t next_nodes, cudaStream_t st);
 int launch_treeimp(const Dev& d, int grid, cudaStream_t st);
 int launch_permut(const Dev& d, int grid, int walk_grid, int sms, cudaStream_t st);
 // walks.cu: the walks, with records of ldP bytes (0: too long) in shared memory, on `st`

@@ -292,9 +292,9 @@ __global__ void k_count(Dev d, int level) {
   if (threadIdx.x == 0) d.chunk[blockIdx.x] = tot;
 }
 
-// The children also go to the next level's lists.  self: the blocks count the
-// level's splits themselves (few nodes: less than a k_count launch).
-__global__ void k_children(Dev d, int level, int self) {
+// list: the children also go to the next level's lists.  self: the blocks count
+// the level's splits themselves (few nodes: less than a k_count launch).
+__global__ void k_children(Dev d, int level, int self, int list) {
   __shared__ uint32_t sw[33];
   __shared__ uint32_t sred[256];
   const uint32_t n = d.lvl_cnt[level], off = d.lvl_off[level];
@@ -388,19 +388,20 @@ __global__ void k_children(Dev d, int level, int self) {
       d.nd_delta[L] = 0.0;
       d.nd_delta[R] = 0.0;
     }
-    if (level + 1 < d.D) list_pair(d, level + 1, cls_l, cls_r, child);
+    if (list) list_pair(d, level + 1, cls_l, cls_r, child);
     run += tot;
   }
 }
 
-// nodes: at most so many at the level
-int launch_children(const Dev& d, int level, uint64_t nodes, cudaStream_t st) {
+// nodes, next_nodes: at most so many at the level and at the next one
+int launch_children(const Dev& d, int level, uint64_t nodes, uint64_t next_nodes, cudaStream_t st) {
+  const int list = level + 1 < d.D && !lists_apart(d.kind != 0, d.three_bins != 0, d.reg_rows != 0, next_nodes);
   if (nodes <= 16384u) {
-    k_children<<<static_cast<unsigned>((nodes + 511u) / 512u), 256, 0, st>>>(d, level, 1);
+    k_children<<<static_cast<unsigned>((nodes + 511u) / 512u), 256, 0, st>>>(d, level, 1, list);
     return 1;
   }
   k_count<<<kScanBlocks, 256, 0, st>>>(d, level);
-  k_children<<<kScanBlocks, 256, 0, st>>>(d, level, 0);
+  k_children<<<kScanBlocks, 256, 0, st>>>(d, level, 0, list);
   return 2;
 }
 

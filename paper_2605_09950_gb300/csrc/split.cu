@@ -215,7 +215,8 @@ __device__ void small_feature(const NodeInfo<1>& nd, int B, bool v, uint32_t b, 
 }
 
 // The lists of the first level, one thread per root: leaves are marked, active
-// nodes listed.  (The later levels' lists are written with their nodes.)
+// nodes listed.  The later levels' lists are written with their nodes, or here
+// (lists_apart).
 template <int KIND, int CM>
 __global__ void __launch_bounds__(256) k_classify(Dev d, int level) {
   const uint32_t lcount = d.lvl_cnt[level], loff = d.lvl_off[level];
@@ -1485,7 +1486,7 @@ int launch_level(const Dev& d, int level, int grid_small, int grid_items, const 
                  uint64_t big_bound, size_t smem, cudaStream_t st, cudaStream_t st2, cudaEvent_t fork, cudaEvent_t join, cudaEvent_t hist_start,
                  cudaEvent_t hist_end) {
   int n = 0;
-  if (level == 0) {
+  if (level == 0 || lists_apart(KIND == 1, d.three_bins != 0, d.reg_rows != 0, nodes)) {
     k_classify<KIND, CM><<<grid_small, 256, 0, st>>>(d, level);
     ++n;
   }

@@ -2,7 +2,7 @@
 with the rows and the sampled columns (reg_record_pays, reg_rows_pays): nodes of
 33 to 1024 rows by blocks or by the column gathers, nodes of at most 32 rows by
 matrix products or by row; genotype columns on both sides of three_bins_pay;
-every tree against the CPU oracle, bit for bit."""
+levels of many nodes, whose lists a kernel of their own writes; trees against the CPU oracle, bit for bit."""
 import numpy as np
 import pytest
 
@@ -38,3 +38,14 @@ def test_three_bin_routes(N, p, bins, n_trees, depth, tie_break):
     y = X[0, :N].astype(np.int64) * 2**20 - X[7, :N].astype(np.int64) * 2**19 + rng.integers(-2**21, 2**21, N)
     w = synth.Workload("t", X, y, N, p, synth.REGRESSION | synth.TREEIMP, 1, bins, n_trees, depth, 2, seed=N, mtry=0)
     check_iteration(w, trees=[0, n_trees - 1], tie_break=tie_break)
+
+
+@pytest.mark.parametrize("N,mtry,n_trees,depth", [(700, 9, 130, 9), (3000, 12, 64, 10)])
+def test_levels_of_many_nodes(N, mtry, n_trees, depth):
+    p, bins = 30, 64
+    rng = np.random.default_rng(N)
+    X = np.zeros((p, synth.pad16(N)), np.uint8)
+    X[:, :N] = rng.integers(0, bins, size=(p, N))
+    y = X[0, :N].astype(np.int64) * 2**17 + rng.integers(-2**21, 2**21, N)
+    w = synth.Workload("t", X, y, N, p, synth.REGRESSION | synth.TREEIMP, 1, bins, n_trees, depth, 2, seed=N, mtry=mtry)
+    check_iteration(w, trees=[0, 1, n_trees - 1])

@@ -84,3 +84,13 @@ THREE_BINS = [("three_bins_pay(20000, 100, 3335, 10006)", 1), ("three_bins_pay(1
 
 def test_three_bins(tmp_path):
     check(tmp_path, THREE_BINS)
+
+
+# lists_apart(regression, three_bins, reg_rows, nodes)
+LISTS = [("lists_apart(true, false, true, 25600)", 1), ("lists_apart(true, false, true, 16384)", 0),
+         ("lists_apart(true, false, false, 10)", 1), ("lists_apart(true, true, false, 25600)", 0),
+         ("lists_apart(false, false, false, 25600)", 0)]
+
+
+def test_lists(tmp_path):
+    check(tmp_path, LISTS)
