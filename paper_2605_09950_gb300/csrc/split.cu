@@ -151,7 +151,7 @@ __device__ void small_feature(const NodeInfo<1>& nd, int B, bool v, uint32_t b, 
       sf[t] = -1.0f;
       nLt[t] = 0u;
       SLt[t] = 0;
-      if (t >= B - 1) break;  // uniform
+      if (t >= B - 1) continue;  // uniform; every threshold's score is set
       const bool in = v && b <= static_cast<uint32_t>(t);
       const uint32_t nl = seg_sum_u32<SEG>(in ? w : 0u);
       const long long sl = seg_sum_i64<SEG>(in ? static_cast<long long>(w) * yv : 0ll);
