@@ -428,6 +428,7 @@ static int session_init(boruta_session* s, const uint8_t* X, int64_t ld, const v
     if ((rc = s->alloc(&d.band_cnt, kMaxBands + 1))) return rc;
   }
   (void)Cmax;
+  size_t table_values = 0;  // leaf values of Alg. 3 as printed
   if (d.permut_form == 1) {
     // Alg. 3 as printed: per row the exact base sums; per block of rows the
     // exact (row, column) deltas, blocks sized to about 1 GiB
@@ -436,11 +437,11 @@ static int session_init(boruta_session* s, const uint8_t* X, int64_t ld, const v
     d.frows = static_cast<uint32_t>(std::max<int64_t>(1, std::min<int64_t>(N, (int64_t{1} << 30) / per_row)));
     if (o->forest_rows > 0) d.frows = std::min<uint32_t>(d.frows, static_cast<uint32_t>(o->forest_rows));
     if ((rc = s->alloc(&d.fbase, static_cast<size_t>(N) * K * kCsaLimbs))) return rc;
-    if ((rc = s->alloc(&d.nd_value, P * K))) return rc;
     if ((rc = s->alloc(&d.fbase_mean, static_cast<size_t>(N) * K))) return rc;
     if ((rc = s->alloc(&d.facc, static_cast<size_t>(d.frows) * p_aug_max * K * kCsaLimbs))) return rc;
     CK(cudaMemsetAsync(d.facc, 0, static_cast<size_t>(d.frows) * p_aug_max * K * kCsaLimbs * sizeof(long long),
                        s->st));
+    table_values = static_cast<size_t>(K) * P;
   }
   CK(cudaMemsetAsync(d.status, 0, 4 * sizeof(uint32_t), s->st));
 
@@ -493,6 +494,9 @@ static int session_init(boruta_session* s, const uint8_t* X, int64_t ld, const v
   CK(cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming));
   CK(cudaEventCreateWithFlags(&s->join, cudaEventDisableTiming));
   s->state_h.assign(p, 0);
+  // last, once all that the session needs is there: without room for the leaf
+  // values the walks divide them themselves
+  if (table_values > 0 && s->alloc(&d.nd_value, table_values)) d.nd_value = nullptr;
   return 0;
 }
 

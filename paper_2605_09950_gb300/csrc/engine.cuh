@@ -100,7 +100,7 @@ struct Dev {
   uint32_t* status;              // [0] error flags, [1] undecided count, [2] n_classes seen
   // ---- Alg. 3 as printed (permut_form = 1)
   long long* fbase;              // [N][K][kCsaLimbs] exact sum over trees of each row's leaf value
-  double* nd_value;              // [cap][K] a node's class fractions, or its mean
+  double* nd_value;              // [cap][K] a node's class fractions, or its mean (null: no room for them)
   double* fbase_mean;            // [N][K] the forest's prediction (K = C, or 1 for regression)
   long long* facc;               // [frows][p_aug][K][kCsaLimbs] per (row of the block, column) delta
   uint32_t frows;                // rows per block

@@ -748,22 +748,25 @@ const void* permut_kernel_ptr(int precision) {
 // permuted prediction.  Each mean is that exact sum rounded once, then
 // divided by M (IEEE), and the per-row losses are summed exactly per column.
 
+__device__ __forceinline__ double divided_value(const Dev& d, int64_t q, int k) {
+  const double n = static_cast<double>(d.nd_n[q]);
+  return d.kind != 0 ? static_cast<double>(d.nd_S[q]) / n : static_cast<double>(d.nd_cnt[q * d.C + k]) / n;
+}
+
 // Each node's value per class, divided once: the walks below read it for every
 // changed leaf, and GB300's FP64 divisions would bind them (N = 5003, 100
-// trees: 1.37 -> 0.24 ms).
+// trees: 1.37 -> 0.24 ms).  Where the memory does not hold the table (nd_value
+// is null) they divide.
 __global__ void k_leaf_values(Dev d) {
   const int K = d.kind != 0 ? 1 : d.C;
   const int64_t total = static_cast<int64_t>(d.lvl_off[d.D] + d.lvl_cnt[d.D]) * K;
   for (int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; t < total;
-       t += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int64_t q = t / K;
-    const int k = static_cast<int>(t - q * K);
-    const double n = static_cast<double>(d.nd_n[q]);
-    d.nd_value[t] = d.kind != 0 ? static_cast<double>(d.nd_S[q]) / n : static_cast<double>(d.nd_cnt[q * d.C + k]) / n;
-  }
+       t += static_cast<int64_t>(gridDim.x) * blockDim.x)
+    d.nd_value[t] = divided_value(d, t / K, static_cast<int>(t % K));
 }
 
 __device__ __forceinline__ double leaf_value(const Dev& d, uint32_t q, int k) {
+  if (!d.nd_value) return divided_value(d, q, k);
   return d.nd_value[static_cast<int64_t>(q) * (d.kind != 0 ? 1 : d.C) + k];
 }
 
@@ -917,11 +920,14 @@ int launch_forest_permut(const Dev& d, int grid, cudaStream_t st) {
   int n = 0;
   k_permut_pi<<<(d.N + 255) / 256 < 1024 ? (d.N + 255) / 256 : 1024, 256, 0, st>>>(d);
   k_pack_nodes<<<grid, 256, 0, st>>>(d);
-  k_leaf_values<<<grid, 256, 0, st>>>(d);
+  if (d.nd_value) {
+    k_leaf_values<<<grid, 256, 0, st>>>(d);
+    ++n;
+  }
   cudaMemsetAsync(d.fbase, 0, static_cast<size_t>(d.N) * forest_k(d) * kCsaLimbs * sizeof(long long), st);
   k_fperm_base<<<grid, 256, 0, st>>>(d);
   k_fperm_base_mean<<<grid, 256, 0, st>>>(d);
-  n += 5;
+  n += 4;
   for (uint32_t r0 = 0; r0 < static_cast<uint32_t>(d.N); r0 += d.frows) {
     const uint32_t rows = min(d.frows, static_cast<uint32_t>(d.N) - r0);
     k_fperm_delta<<<grid, 256, 0, st>>>(d, r0, rows);
