@@ -765,8 +765,11 @@ __global__ void k_leaf_values(Dev d) {
     d.nd_value[t] = divided_value(d, t / K, static_cast<int>(t % K));
 }
 
+// TABLE: whether nd_value is there (a template argument: the divisions'
+// registers would cost the other form 12% of its time)
+template <bool TABLE>
 __device__ __forceinline__ double leaf_value(const Dev& d, uint32_t q, int k) {
-  if (!d.nd_value) return divided_value(d, q, k);
+  if (!TABLE) return divided_value(d, q, k);
   return d.nd_value[static_cast<int64_t>(q) * (d.kind != 0 ? 1 : d.C) + k];
 }
 
@@ -789,6 +792,7 @@ __device__ __forceinline__ uint32_t forest_walk(const Dev& d, uint32_t k, uint32
 __host__ __device__ __forceinline__ int forest_k(const Dev& d) { return d.kind != 0 ? 1 : d.C; }
 
 // one thread per (tree, row): the row's leaf value into its exact base sum
+template <bool TABLE>
 __global__ void k_fperm_base(Dev d) {
   const int K = forest_k(d);
   const int64_t items = static_cast<int64_t>(d.M) * d.N;
@@ -798,7 +802,7 @@ __global__ void k_fperm_base(Dev d) {
     const uint32_t i = static_cast<uint32_t>(it - static_cast<int64_t>(tau) * d.N);
     const uint32_t q = forest_walk(d, static_cast<uint32_t>(tau), i, 0xFFFFFFFFu, 0u);
     for (int k = 0; k < K; ++k)
-      if (!csa_add(d.fbase + (static_cast<int64_t>(i) * K + k) * kCsaLimbs, leaf_value(d, q, k)))
+      if (!csa_add(d.fbase + (static_cast<int64_t>(i) * K + k) * kCsaLimbs, leaf_value<TABLE>(d, q, k)))
         atomicOr(&d.status[0], kErrAcc);
   }
 }
@@ -819,6 +823,7 @@ __global__ void k_fperm_base_mean(Dev d) {
 // column f on it, the leaf reached with f read at flush_index (the walk
 // leaves the path at the first node testing f that sends the swapped value
 // the other way); a changed leaf adds (new - old) per class to (row, f).
+template <bool TABLE>
 __global__ void k_fperm_delta(Dev d, uint32_t r0, uint32_t rows) {
   const int K = forest_k(d);
   const int64_t items = static_cast<int64_t>(d.M) * rows;
@@ -862,7 +867,7 @@ __global__ void k_fperm_delta(Dev d, uint32_t r0, uint32_t rows) {
       long long* acc = d.facc + ((static_cast<int64_t>(loc) * d.p_aug + f) * K) * kCsaLimbs;
       bool ok = true;
       for (int c = 0; c < K; ++c)
-        ok &= csa_add_diff(acc + c * kCsaLimbs, leaf_value(d, q2, c), leaf_value(d, q, c));
+        ok &= csa_add_diff(acc + c * kCsaLimbs, leaf_value<TABLE>(d, q2, c), leaf_value<TABLE>(d, q, c));
       if (!ok) atomicOr(&d.status[0], kErrAcc);
     }
   }
@@ -920,17 +925,24 @@ int launch_forest_permut(const Dev& d, int grid, cudaStream_t st) {
   int n = 0;
   k_permut_pi<<<(d.N + 255) / 256 < 1024 ? (d.N + 255) / 256 : 1024, 256, 0, st>>>(d);
   k_pack_nodes<<<grid, 256, 0, st>>>(d);
-  if (d.nd_value) {
+  const bool table = d.nd_value != nullptr;
+  if (table) {
     k_leaf_values<<<grid, 256, 0, st>>>(d);
     ++n;
   }
   cudaMemsetAsync(d.fbase, 0, static_cast<size_t>(d.N) * forest_k(d) * kCsaLimbs * sizeof(long long), st);
-  k_fperm_base<<<grid, 256, 0, st>>>(d);
+  if (table)
+    k_fperm_base<true><<<grid, 256, 0, st>>>(d);
+  else
+    k_fperm_base<false><<<grid, 256, 0, st>>>(d);
   k_fperm_base_mean<<<grid, 256, 0, st>>>(d);
   n += 4;
   for (uint32_t r0 = 0; r0 < static_cast<uint32_t>(d.N); r0 += d.frows) {
     const uint32_t rows = min(d.frows, static_cast<uint32_t>(d.N) - r0);
-    k_fperm_delta<<<grid, 256, 0, st>>>(d, r0, rows);
+    if (table)
+      k_fperm_delta<true><<<grid, 256, 0, st>>>(d, r0, rows);
+    else
+      k_fperm_delta<false><<<grid, 256, 0, st>>>(d, r0, rows);
     k_fperm_loss<<<grid, 256, 0, st>>>(d, r0, rows);
     n += 2;
   }
