@@ -295,10 +295,6 @@ static int session_init(boruta_session* s, const uint8_t* X, int64_t ld, const v
   if ((rc = s->alloc(&d.nd_split, P))) return rc;
   if ((rc = s->alloc(&d.nd_child, P))) return rc;
   if (d.permut && (rc = s->alloc(&d.nd_sc, P))) return rc;
-  if (d.permut && d.permut_form == 0 && use_walks(d)) {
-    if ((rc = s->alloc(&d.wt_tree, n_trees + 1))) return rc;
-    CK(static_cast<cudaError_t>(setup_walks()));
-  }
   if ((rc = s->alloc(&d.nd_delta, P))) return rc;
   if ((rc = s->alloc(&d.nd_lrows, P))) return rc;
   if ((rc = s->alloc(&d.nd_ln, P))) return rc;
@@ -381,6 +377,10 @@ static int session_init(boruta_session* s, const uint8_t* X, int64_t ld, const v
   if (!reg) {
     if ((rc = s->alloc(&d.nd_cnt, P * d.C))) return rc;
     if ((rc = s->alloc(&d.nd_lcnt, P * d.C))) return rc;
+  }
+  if (d.permut && d.permut_form == 0 && use_walks(d)) {  // (the rule asks for the classes)
+    if ((rc = s->alloc(&d.wt_tree, n_trees + 1))) return rc;
+    CK(static_cast<cudaError_t>(setup_walks()));
   }
   // larger nodes of one level: at most N/33 per tree (each has > 32 rows), or
   // N/65 for classification (> 64 rows; mid nodes: N/33 of > 32 rows, and N/67
@@ -535,7 +535,7 @@ int boruta_session_create(const uint8_t* X, int64_t ld, const void* y, int64_t N
 // columns or trees they do not pay (records_pay).  Columns of at most 4 bins stay
 // with the register counts of the column path.
 static uint32_t record_rows(const boruta_session* s, const Dev& d) {
-  if (d.kind != 0 || s->split_path != 0 || d.B <= 4 || !records_pay(d.N, d.M, d.mtry)) return 0u;
+  if (d.kind != 0 || s->split_path != 0 || d.B <= 4 || !records_pay(d.N, d.M, d.mtry, d.D, d.C)) return 0u;
   const bool in_l2 = static_cast<uint64_t>(d.N) * static_cast<uint64_t>(d.ldP) <= (96ull << 20);
   return std::min<uint32_t>(kRecordRows, static_cast<uint32_t>(d.N) / (in_l2 ? 1u : 64u));
 }
@@ -549,7 +549,7 @@ static uint32_t record_rows(const boruta_session* s, const Dev& d) {
 // record.cu holds every node in one launch.
 static int32_t use_columns(const boruta_session* s, const Dev& d) {
   if (d.kind != 0 || s->split_path != 0 || s->col_grid == 0 || d.B <= 4) return 0;
-  if (d.N <= static_cast<int32_t>(kRecordRows) || !columns_pay(d.N, d.M, d.mtry)) return 0;
+  if (d.N <= static_cast<int32_t>(kRecordRows) || !columns_pay(d.N, d.M, d.mtry, d.D, d.C)) return 0;
   const uint64_t nodes = static_cast<uint64_t>(d.M) * (static_cast<uint64_t>(d.N) / 257 + 1);
   return nodes * static_cast<uint64_t>(d.mtry) <= d.item_cap;
 }

@@ -52,17 +52,21 @@ struct Dev {
   uint2* wt_tree;                // [M + 1] walks.cu: a tree's first packed split node and their number; the total
   uint32_t* work;                // [D + 2] per level: number of nodes in `big`
   uint32_t* chunk;               // [kScanBlocks] per-block split counts
-  uint32_t* big;                 // [big_cap] this level's active nodes of more rows than the lists below
-  uint32_t* small;               // [level_cap] this level's active nodes with <= 32 rows
-  uint32_t* nsmall;              // [D + 2] per level: number of 17..32-row nodes at the start of `small`
+  uint32_t* big;                 // [big_cap] this level's active nodes of the column gathers
+  uint32_t* small;               // [level_cap] this level's active nodes of 9..32 rows (three_bins: of 9 to 16383)
+  uint32_t* nsmall;              // [D + 2] per level: number of 17..32-row nodes (three_bins: of all) at the
+                                 //   start of `small`
   uint32_t* ntiny;               // [D + 2] per level: number of 9..16-row nodes at the end of `small`
   uint32_t* micro;               // [small_cap] this level's active nodes with <= 8 rows
   uint32_t* nmicro;              // [D + 2] per level: number of them
   uint32_t* mid;                 // [mid_cap] classification: nodes of 33..64 rows, and smaller ones
                                  //   whose weight exceeds kFewWeight
   uint32_t* nmid;                // [D + 2] per level: number of them
-  uint32_t* rec;                 // nodes split by record: of 65..256 rows (record.cu), 33..256 (regress.cu)
-  uint32_t* rec2;                // [rec2_cap] of 257..1024 rows (from its start), of up to 4096 (from its end)
+  uint32_t* rec;                 // nodes split by record: of 65..256 rows and weight below 1024 (record.cu),
+                                 //   of 33..256 rows (regress.cu)
+  uint32_t* rec2;                // [rec2_cap] from its start: of 257..1024 rows (record.cu: and smaller ones of
+                                 //   weight 1024..4095; `columns`: the nodes of column.cu, of any size above);
+                                 //   from its end: record.cu's nodes of up to 4096 rows
   uint32_t* nrec;                // [D + 2][3] per level: numbers of the three
   uint32_t rec2_cap;
   uint32_t rec_rows;             // largest node split by record (0: none)
@@ -177,7 +181,7 @@ int launch_children(const Dev& d, int level, uint64_t nodes, uint64_t next_nodes
 int launch_treeimp(const Dev& d, int grid, cudaStream_t st);
 int launch_permut(const Dev& d, int grid, int walk_grid, int sms, cudaStream_t st);
 // walks.cu: the walks, with records of ldP bytes (0: too long) in shared memory, on `st`
-inline bool use_walks(const Dev& d) { return walks_pay(d.kind == 0, d.precision != 0, d.N, d.M, d.D); }
+inline bool use_walks(const Dev& d) { return walks_pay(d.kind == 0 ? d.C : 0, d.precision != 0, d.N, d.M, d.D); }
 uint32_t walk_nodes(int D, int ldP);
 int setup_walks();
 int launch_walks(const Dev& d, int sms, cudaStream_t st);  // Dev::nd_sc, nd_ln, nd_lrows, nd_lcnt are its scratch

@@ -712,7 +712,7 @@ __global__ void k_permut_final(Dev d) {
 int launch_permut(const Dev& d, int grid, int walk_grid, int sms, cudaStream_t st) {
   k_permut_pi<<<(d.N + 255) / 256 < 1024 ? (d.N + 255) / 256 : 1024, 256, 0, st>>>(d);
   int n = 4;
-  if (use_walks(d) && walk_nodes(d.D, d.ldP) > 0u) {
+  if (d.wt_tree && walk_nodes(d.D, d.ldP) > 0u) {  // (wt_tree: use_walks)
     n = 2 + launch_walks(d, sms, st);
   } else {
     k_pack_nodes<<<grid, 256, 0, st>>>(d);

@@ -6,9 +6,10 @@
 namespace bgb {
 
 // Alg. 3 by walks.cu (else k_permut).  Packing the trees and filling shared
-// memory pays for large forests of deep trees only, and only while a re-walk's
-// loss is cheap: its 3 rows a warp leave half the lanes of the loss idle, which
-// the FP64 units (divisions and a logarithm per class) cannot hide.
+// memory pays for large forests of deep trees, and only while a re-walk's loss
+// is cheap: its 3 rows a warp leave half the lanes of the loss idle, which the
+// FP64 units (divisions and a logarithm per class) cannot hide.  The rows of all
+// trees that it takes grow by half with every level below 17.
 // Importance stage, k_permut -> walks.cu, ms:
 //   FP32 terms, 2 / 5 / 8 classes
 //     N = 8192, 100 trees, depth 16        0.25 -> 0.38, 0.33 -> 0.43, 0.36 -> 0.47
@@ -17,16 +18,25 @@ namespace bgb {
 //     N = 50000, 100 trees, depth 12       0.88 -> 1.10, 1.25 -> 1.25, 1.44 -> 1.35
 //     N = 50000, 100 trees, depth 16       1.40 -> 1.33, 1.97 -> 1.53, 2.27 -> 1.67
 //     N = 1e5, 100 trees, depth 20         4.23 -> 2.99, 6.52 -> 3.42, 7.51 -> 3.80
+//   times as fast at N x trees (1e6), over 150 random problems: depth 13 0.96 at
+//   4.0, 1.04 at 6.1, 1.2 at 12 to 27; depth 15 0.9 at 1.5, 1.04 at 4.4, 1.3 at 10 to
+//   31; depth 17 0.95 at 2.7, 1.2 at 4, 1.7 at 10 to 26; depth 19 and 20 0.9 at 1.1, 1.3
+//   at 2 to 4, 1.7 at 16 to 53; two classes 0.7 to 1.0 at 1.4 to 20 below depth 15
 //   FP64 terms: 2 to 25 times the time of k_permut everywhere measured
 //     N = 1e5, 100 trees, depth 20         7.38 -> 14.2, 18.9 -> 35.5, 29.3 -> 56.4
 //   regression (FP64 / FP32 terms)
 //     N = 20000, 100 trees, depth 16       0.65 -> 0.73, 0.63 -> 0.64
 //     N = 1e5, 100 trees, depth 16         3.57 -> 3.04, 3.46 -> 2.68
-inline bool walks_pay(bool classification, bool fp32, int64_t N, int64_t trees, int depth) {
-  if (N < 8192 || depth < 16) return false;
+// classes: 0 for regression
+inline bool walks_pay(int classes, bool fp32, int64_t N, int64_t trees, int depth) {
+  if (N < 8192 || depth < 12) return false;
   const int64_t rows = N * trees;
-  if (!classification) return rows >= 10000000;
-  return fp32 && rows >= (depth < 20 ? 5000000 : 2000000);
+  if (classes == 0) return depth >= 16 && rows >= 10000000;
+  if (!fp32) return false;
+  int64_t need = depth >= 19 ? 1500000 : 2000000;
+  for (int l = 17; l > depth; --l) need += need / 2;
+  if (classes <= 2 && depth < 15) need *= 2;
+  return rows >= need;
 }
 
 // Classification nodes above 64 rows in problems of 65,536 rows and more, whose
@@ -35,8 +45,9 @@ inline bool walks_pay(bool classification, bool fp32, int64_t N, int64_t trees, 
 // every level, and the longest node of each is waited for in turn; with few
 // (node, column) items, which leave the GPU idle, the bands alone take all the
 // nodes of a level together in less time.  Both lines by the columns a node
-// samples and the trees; below 65,536 rows (and a little above, where few
-// levels hold both) there is no second wait, and the rules say yes.
+// samples, the trees and the depth (few rows a node, and many nodes, lie deep);
+// below 65,536 rows (and a little above, where few levels hold both) there is no
+// second wait, and the rules say yes.
 // Split stage, column.cu against the bands alone, times as fast (2, 5 classes,
 // depth 12):
 //   N = 60000, 30 trees, 10 / 31 columns      2.20, 1.49 / 1.95, 1.61
@@ -45,9 +56,17 @@ inline bool walks_pay(bool classification, bool fp32, int64_t N, int64_t trees, 
 //   N = 1e5, 30 trees, 10 / 31 / 63           0.97, 0.91 / 0.95, 0.89 / 1.24, 1.10
 //   N = 1e5, 200 trees, 4 / 20 / 44           0.85, 0.80 / 1.03, 1.05 / 1.37, 1.22
 //   N = 130000, 60 trees, 10 / 31 / 63        0.82, 0.78 / 0.92, 0.86 / 1.22, 1.13
-inline bool columns_pay(int64_t N, int64_t trees, int64_t mtry) {
-  if (N < (mtry >= 8 ? 81920 : 72000) || mtry >= 44 || trees <= 3) return true;
-  return 14 * trees * mtry >= N - 65536;
+// Over 500 problems of 2 to 8 classes and 32 to 256 bins: from depth 13 on columns
+// win with a tenth of the items (column, tree) that they need at depth 9 to 12, up
+// to depth 8 only where there are many (N = 75,000 to 120,000, 3000 to 5500 items
+// 1.08 to 1.28 times as fast, 400 to 2000 0.81 to 0.99); six and more classes, whose
+// histograms hold three and four words a bin, need as many as depth 9 to 12.
+inline bool columns_pay(int64_t N, int64_t trees, int64_t mtry, int depth, int classes) {
+  if (N < 66000 || trees <= 3) return true;
+  const int64_t items = trees * mtry;
+  if (depth <= 8) return items >= 2300 && 16 * items >= N - 65536;
+  if (N < 82000 || (mtry >= 44 && N < 110000)) return true;
+  return (classes >= 6 ? 16 : (depth > 12 ? 200 : 28)) * items >= N - 65536;
 }
 
 // record.cu (where column.cu does not take the problem) against the bands alone,
@@ -56,8 +75,14 @@ inline bool columns_pay(int64_t N, int64_t trees, int64_t mtry) {
 //   N = 2e5, depth 12, 10 trees                             0.87 / 0.86 / 0.92 / 1.07
 //   N = 2e5, depth 20, 100 trees                            0.78 / 0.89 / 1.18 / 1.35
 //   N = 1e6, depth 20, 300 trees, 10 / 31 columns           0.87 / 1.15
-inline bool records_pay(int64_t N, int64_t trees, int64_t mtry) {
-  return N < 65536 || mtry >= 48 || (mtry >= 24 && trees * mtry >= 900);
+//   N = 2e5, 2 classes, 14 to 26 columns, 266 to 362 trees, depth 11 to 18  1.02 to 1.12
+//   N = 2e5, 6 classes, 33 columns, 132 trees, depth 10     0.88
+inline bool records_pay(int64_t N, int64_t trees, int64_t mtry, int depth, int classes) {
+  if (N < 65536) return true;
+  if (depth <= 9) return false;
+  const int64_t items = trees * mtry;
+  if (mtry >= 60 || (classes <= 2 && mtry >= 14 && depth >= 11 && items >= 2500)) return true;
+  return mtry >= 22 && items >= (depth <= 13 ? 2300 : 900);
 }
 
 // Regression over more than 4 bins.  Nodes of 33..1024 rows by regress.cu's

@@ -18,7 +18,8 @@ pytestmark = pytest.mark.gpu
     (8300, 1024, 2, 16, 20, 9, 2_000_000, 1),   # records of 2048 bytes, the longest staged
     (8300, 1030, 2, 16, 20, 9, 2_000_000, 1),   # longer
     (60_001, 1000, 8, 256, 30, 2, 2_000_000, 1),  # more split nodes than fit beside records of 2000 bytes
-    (9003, 40, 5, 256, 16, 6, 5_000_000, 1),
+    (9003, 40, 5, 256, 16, 6, 3_000_000, 1),
+    (9003, 40, 8, 256, 14, 6, 6_750_000, 1),
     (50_001, 20, 1, 128, 16, 10, 10_000_000, 0),  # regression
     (50_001, 20, 1, 128, 16, 10, 10_000_000, 1),
 ])

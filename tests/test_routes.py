@@ -21,35 +21,43 @@ def check(where, cases):
     assert [(e, g) for (e, _), g in zip(cases, got)] == [(e, int(want)) for e, want in cases]
 
 
-# walks_pay(classification, fp32, N, trees, depth)
-WALKS = [("walks_pay(true, true, 1000000, 300, 20)", 1), ("walks_pay(true, true, 100000, 500, 16)", 1),
-         ("walks_pay(true, true, 100000, 100, 20)", 1), ("walks_pay(true, true, 20000, 100, 20)", 1),
+# walks_pay(classes (0: regression), fp32, N, trees, depth)
+WALKS = [("walks_pay(5, true, 1000000, 300, 20)", 1), ("walks_pay(2, true, 100000, 500, 16)", 1),
+         ("walks_pay(5, true, 100000, 100, 20)", 1), ("walks_pay(2, true, 20000, 100, 20)", 1),
+         ("walks_pay(8, true, 90320, 224, 12)", 1), ("walks_pay(4, true, 166321, 160, 13)", 1),
          # few trees, few rows: one block after another
-         ("walks_pay(true, true, 8192, 1, 20)", 0), ("walks_pay(true, true, 8192, 100, 16)", 0),
-         ("walks_pay(true, true, 100000, 10, 16)", 0), ("walks_pay(true, true, 8191, 100000, 20)", 0),
+         ("walks_pay(5, true, 8192, 1, 20)", 0), ("walks_pay(8, true, 8192, 100, 16)", 0),
+         ("walks_pay(8, true, 100000, 10, 16)", 0), ("walks_pay(5, true, 8191, 100000, 20)", 0),
          # trees of few levels
-         ("walks_pay(true, true, 1000000, 300, 12)", 0),
+         ("walks_pay(2, true, 198838, 99, 12)", 0), ("walks_pay(5, true, 130989, 265, 11)", 0),
+         ("walks_pay(2, true, 14753, 172, 14)", 0),
          # FP64 losses of classes, at any size
-         ("walks_pay(true, false, 1000000, 300, 20)", 0), ("walks_pay(true, false, 100000, 100, 16)", 0),
+         ("walks_pay(5, false, 1000000, 300, 20)", 0), ("walks_pay(2, false, 100000, 100, 16)", 0),
          # regression
-         ("walks_pay(false, false, 100000, 100, 16)", 1), ("walks_pay(false, true, 20000, 100, 16)", 0),
-         ("walks_pay(false, false, 10000, 100, 16)", 0)]
+         ("walks_pay(0, false, 100000, 100, 16)", 1), ("walks_pay(0, true, 20000, 100, 16)", 0),
+         ("walks_pay(0, false, 10000, 100, 16)", 0)]
 
 
 def test_walks(tmp_path):
     check(tmp_path, WALKS)
 
 
-# columns_pay(N, trees, mtry), records_pay(N, trees, mtry)
+# columns_pay(N, trees, mtry, depth, classes), records_pay(N, trees, mtry, depth, classes)
 LARGE_CLASSIFICATION = [
-    ("columns_pay(30011, 100, 20)", 1), ("columns_pay(65535, 1, 1)", 1), ("columns_pay(66000, 200, 4)", 1),
-    ("columns_pay(80000, 200, 4)", 0), ("columns_pay(80000, 60, 31)", 1),
-    ("columns_pay(100000, 500, 44)", 1), ("columns_pay(100000, 200, 31)", 1), ("columns_pay(100000, 1, 4)", 1),
-    ("columns_pay(100000, 30, 31)", 0), ("columns_pay(100000, 100, 10)", 0), ("columns_pay(100000, 200, 4)", 0),
-    ("columns_pay(130000, 60, 31)", 0), ("columns_pay(130000, 200, 10)", 0), ("columns_pay(130000, 200, 44)", 1),
-    ("records_pay(4000, 1, 1)", 1), ("records_pay(1000000, 300, 31)", 1), ("records_pay(200000, 100, 31)", 1),
-    ("records_pay(200000, 10, 63)", 1), ("records_pay(200000, 100, 10)", 0), ("records_pay(400000, 300, 10)", 0),
-    ("records_pay(1000000, 10, 14)", 0), ("records_pay(400000, 10, 20)", 0)]
+    ("columns_pay(30011, 100, 20, 14, 5)", 1), ("columns_pay(65535, 1, 1, 4, 5)", 1), ("columns_pay(80000, 60, 31, 12, 5)", 1),
+    ("columns_pay(85895, 74, 7, 18, 5)", 1), ("columns_pay(100000, 500, 44, 16, 5)", 1), ("columns_pay(100000, 200, 31, 12, 5)", 1),
+    ("columns_pay(100000, 1, 4, 12, 5)", 1), ("columns_pay(156675, 302, 22, 18, 5)", 1),
+    ("columns_pay(100000, 30, 31, 12, 5)", 0), ("columns_pay(100000, 100, 10, 12, 5)", 0), ("columns_pay(100000, 200, 4, 12, 5)", 0),
+    ("columns_pay(130000, 60, 31, 12, 5)", 0), ("columns_pay(78669, 33, 39, 6, 5)", 0), ("columns_pay(124008, 110, 13, 7, 5)", 0),
+    ("columns_pay(130000, 200, 44, 12, 5)", 1), ("columns_pay(99934, 46, 37, 11, 2)", 1),
+    ("columns_pay(85282, 99, 42, 6, 5)", 1), ("columns_pay(142259, 89, 43, 6, 2)", 0),
+    ("columns_pay(105741, 39, 14, 15, 6)", 0), ("records_pay(219170, 76, 23, 16, 5)", 1),
+    ("records_pay(4000, 1, 1, 12, 2)", 1), ("records_pay(1000000, 300, 31, 20, 5)", 1),
+    ("records_pay(200000, 100, 31, 12, 5)", 1), ("records_pay(200000, 10, 63, 12, 5)", 1),
+    ("records_pay(215719, 197, 15, 16, 2)", 1), ("records_pay(214267, 266, 21, 18, 2)", 1),
+    ("records_pay(200000, 100, 10, 12, 5)", 0), ("records_pay(400000, 300, 10, 20, 5)", 0),
+    ("records_pay(1000000, 10, 14, 12, 2)", 0), ("records_pay(400000, 10, 20, 12, 5)", 0),
+    ("records_pay(221890, 97, 42, 8, 8)", 0), ("records_pay(225026, 115, 20, 18, 6)", 0)]
 
 
 def test_large_classification(tmp_path):
