@@ -20,7 +20,6 @@ bounded sample of the same workload instead.
 from __future__ import annotations
 
 import argparse
-import hashlib
 import json
 import os
 import statistics
@@ -50,23 +49,6 @@ WORKLOADS = {
     "small": ("binary_small", dict(),
               "Boruta iterations/sec (binary N=1000, p=50, 100 trees, depth 8, impurity importance)", "treeimp"),
 }
-
-# DRAM bytes (read + write) of the larger nodes' split kernels per tree level,
-# from one ncu capture of a whole iteration: workload -> bytes_per_launch,
-# sources_sha16 (valid only while the kernels' and their launch code's sources
-# hash to it), profile.  No capture of the present kernels: the line reports null.
-TRAFFIC = {}
-
-
-def kernel_source_sha16():
-    """Hash of the histogram kernel's sources and of the host code that sets
-    its launches (a recorded traffic figure holds only for these)."""
-    h = hashlib.sha256()
-    for name in ("split.cu", "record.cu", "column.cu", "planes.cuh", "engine.cuh", "api.cu"):
-        with open(os.path.join(ROOT, "paper_2605_09950_gb300", "csrc", name), "rb") as f:
-            h.update(f.read())
-    return h.hexdigest()[:16]
-
 
 def peaks():
     try:
@@ -465,9 +447,6 @@ def run_gpu(args):
     peak, peak_kind = peaks()
     achieved = ks["hist_bytes"] / (ks["hist_ms"] / 1000.0) / 1e9 if ks["hist_ms"] > 0 else 0.0
     split_gbs = ks["split_bytes"] / (ks["split_ms"] / 1000.0) / 1e9 if ks["split_ms"] > 0 else 0.0
-    prof = TRAFFIC.get(w.name)
-    traffic = prof["bytes_per_launch"] if prof and prof["sources_sha16"] == kernel_source_sha16() \
-        and not args.trees else None
     permut = importance == "permut_oob"
     walks = None
     if permut and ks["imp_ms"] > 0:
@@ -491,8 +470,8 @@ def run_gpu(args):
                    "l2": "512 MiB buffer written before each timed step; inputs and per-step working set > L2",
                    "input_generation_s": round(gen_s, 1), "session_setup_s": round(setup_s, 2)},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                     "frac": achieved / peak if peak else None, "traffic": traffic,
-                     "traffic_source": prof["profile"] if traffic else None,
+                     "frac": achieved / peak if peak else None,
+                     "traffic": None,  # no counter capture of a whole iteration
                      "kernel": "split kernels of the nodes of more than 64 rows (k_record, k_column, k_items_band; "
                                "regression: k_reg_record, k_three_rows, k_items_band)",
                      "peak_kind": f"{peak_kind} hbm_gbs (burst copy)", "launches": int(ks["launches"]),
