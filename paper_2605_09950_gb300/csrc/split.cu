@@ -3,8 +3,9 @@
 // TreeImp accumulators (Alg. 2) and the stable row partition.
 //
 // Kernels of a level:
-//   k_classify      (first level) leaves, and the lists of active nodes; the
-//                   other levels' lists come with their nodes (k_children).
+//   k_classify      (first level, and regression levels of lists_apart) leaves,
+//                   and the lists of active nodes; the other levels' lists come
+//                   with their nodes (k_children).
 //   small.cu, record.cu, column.cu, regress.cu, threebin.cu take the nodes
 //   that their kernels are made for (lists.cuh); here:
 //   k_split_small   (second stream) regression nodes of at most 32 rows that
@@ -809,8 +810,7 @@ __device__ void scan_pack(const Dev& d, const NodeInfo<CM>& nd, const uint32_t* 
 // class (class k in bits 12k .. 12k+11).  Every partial sum of a bin or of a
 // prefix of bins is at most the node's total weight, so no field carries into
 // the next: one shared-memory add, load, scan step or store moves all the
-// classes of a bin.  Staged nodes (at most kRegRows rows of bootstrap count
-// below 32) always qualify.
+// classes of a bin.
 constexpr int kPkBits = 12;
 constexpr uint32_t kPkLimit = 1u << kPkBits;
 

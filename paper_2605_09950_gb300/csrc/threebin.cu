@@ -1,5 +1,5 @@
 // Split search of regression nodes over columns of at most three bins
-// (genotypes), where a node samples a large share of the columns.
+// (genotypes), where a node samples many of them (three_bins_pay in routes.h).
 //
 // Two thresholds per column, and every threshold's left totals are sums over
 // the node's rows: with Le[(f, b)][s] = 1 where bin_s(f) <= b, the sums for all
