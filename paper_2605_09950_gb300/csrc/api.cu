@@ -579,7 +579,7 @@ static int enqueue_iteration(boruta_session* s, int t, cudaStream_t st) {
   if (d.columns) d.rec_rows = 256;
   const int col_grids[2] = {s->rec_grid[0], s->col_grid};
   d.three_bins = d.kind == 1 && d.B <= 3 && s->split_path == 0 && s->rec_grid[0] > 0 && s->rec_grid[1] > 0 &&
-                 three_bins_pay(d.N, d.M, d.mtry, p_aug);
+                 three_bins_pay(d.N, d.M, d.mtry, p_aug, d.D);
   // regress.cu: columns of more than 4 bins (fewer are counted in registers by
   // the column path), lists of 16-bit columns
   const bool reg_ok = d.kind == 1 && d.B > 4 && s->split_path == 0 && d.mtry <= kRegColumns && p_aug <= 65536;

@@ -122,9 +122,33 @@ inline bool reg_rows_pays(int64_t N, int64_t mtry) { return N <= 2048 || mtry >=
 //   N = 40000, 10 trees, 13 / 50 / 100          0.61 / 0.84 / 1.33 (p = 50)
 //   N = 30000, 100 trees, 40 / 66               0.85 / 1.22 (p = 60, 100; iteration)
 //   N = 40000, 1 tree, 500 / 1000 of 4000       0.66 / 1.21
-// From 16,384 rows on the largest nodes go to the gathers in any case.
-inline bool three_bins_pay(int64_t N, int64_t trees, int64_t mtry, int64_t columns) {
+// From 16,384 rows on the largest nodes go to the gathers in any case.  Shallow
+// trees are few large nodes, a block each, whose time the level waits for, and do
+// not reach the small ones (iteration, times as fast, depth 2 / 4 / 6 / 8):
+//   N = 4000, 10 trees, 133 / 1333 columns     1.12 / 1.69 / 2.65 / 3.56    0.71 / 1.02 / 4.39 / 7.70
+//   N = 8000, 10 trees, 66 / 400               0.78 / 0.97 / 1.31 / 1.65    0.74 / 0.93 / 1.83 / 3.18
+//   N = 8000, 100 trees, 66 / 400              1.08 / 1.09 / 1.36 / 1.47    1.51 / 1.70 / 2.87 / 3.73
+//   N = 16000, 10 trees, 133 / 400             0.63 / 0.73 / 1.04 / 1.48    0.53 / 0.64 / 1.05 / 1.96
+//   N = 16000, 100 trees, 66 / 133             0.89 / 0.84 / 1.04 / 1.23    1.22 / 1.27 / 1.63 / 2.08
+//   N = 70000, depth 4 / 6 / 8 / 10, 30 trees, 66 / 133  0.76 / 0.76 / 0.86 / 1.01, 0.88 / 0.96 / 1.15 / 1.50
+//   N = 200000, the same                       0.89 / 0.82 / 0.84 / 0.95, 0.94 / 0.92 / 1.03 / 1.22
+inline bool three_bins_pay(int64_t N, int64_t trees, int64_t mtry, int64_t columns, int depth) {
   if (8 * mtry < columns || (N >= 16384 && 4 * mtry < columns)) return false;
+  const int64_t items = trees * mtry;
+  if (depth <= 4) {
+    if (N > 8192) {
+      if (items < 12000 || trees < (depth <= 2 ? 100 : 30)) return false;
+    } else if (N > 4096) {
+      if (trees < (depth <= 2 ? 100 : 30)) return false;
+    } else if (depth <= 2 && N > 1024 && trees < 30) {
+      return false;
+    }
+  } else if (depth <= 7) {
+    const bool many = items >= 4000 && trees >= 30 && 15 * items >= N && (N < 16384 || mtry >= 128);
+    if (N > 8192 && !many && !(N < 16384 && trees >= 10 && mtry >= 128)) return false;
+  } else if (N >= 16384 && (depth < 10 ? 30 : (depth < 13 ? 100 : 200)) * items < N) {
+    return false;
+  }
   if (mtry >= 64 || (mtry >= 40 && N <= 5000) || (mtry >= 24 && N <= 1024)) return true;
   return N <= 5000 && N * trees <= (mtry >= 16 ? 200000 : 100000);
 }

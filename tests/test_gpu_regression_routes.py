@@ -30,7 +30,8 @@ def test_regression_routes(N, mtry, bins, depth, tie_break):
 @pytest.mark.parametrize("tie_break", [0, 1])
 @pytest.mark.parametrize("N,p,bins,n_trees,depth", [
     (2500, 20, 3, 40, 9), (2500, 20, 3, 41, 9), (17_001, 60, 3, 4, 6),  # records; by row (13 and 40 columns)
-    (16_400, 150, 3, 2, 5), (27_000, 150, 2, 2, 3)])  # records, and nodes of more than 16383 rows by column
+    (16_400, 150, 3, 2, 13), (27_000, 150, 2, 2, 13),  # records, and nodes of more than 16383 rows by column
+    (16_400, 150, 3, 2, 5), (8200, 70, 3, 3, 2)])  # shallow: by row
 def test_three_bin_routes(N, p, bins, n_trees, depth, tie_break):
     rng = np.random.default_rng(N + p)
     X = np.zeros((p, synth.pad16(N)), np.uint8)

@@ -79,15 +79,21 @@ def test_regression(tmp_path):
     check(tmp_path, REGRESSION)
 
 
-# three_bins_pay(N, trees, mtry, columns)
-THREE_BINS = [("three_bins_pay(20000, 100, 3335, 10006)", 1), ("three_bins_pay(1000, 100, 6, 48)", 1),
-              ("three_bins_pay(5000, 10, 6, 48)", 1), ("three_bins_pay(5000, 100, 133, 400)", 1),
-              ("three_bins_pay(16000, 100, 100, 100)", 1), ("three_bins_pay(40000, 100, 100, 400)", 1),
-              ("three_bins_pay(2000, 100, 16, 48)", 1), ("three_bins_pay(2000, 300, 40, 120)", 1),
-              ("three_bins_pay(30000, 100, 66, 200)", 1), ("three_bins_pay(2000, 300, 16, 48)", 0),
-              ("three_bins_pay(5000, 100, 24, 48)", 0), ("three_bins_pay(16000, 100, 33, 100)", 0),
-              ("three_bins_pay(40000, 10, 33, 100)", 0), ("three_bins_pay(40000, 1, 500, 4000)", 0),
-              ("three_bins_pay(300, 10, 10, 100)", 0)]
+# three_bins_pay(N, trees, mtry, columns, depth)
+THREE_BINS = [("three_bins_pay(20000, 100, 3335, 10006, 10)", 1), ("three_bins_pay(1000, 100, 6, 48, 10)", 1),
+              ("three_bins_pay(5000, 10, 6, 48, 10)", 1), ("three_bins_pay(5000, 100, 133, 400, 10)", 1),
+              ("three_bins_pay(16000, 100, 100, 100, 10)", 1), ("three_bins_pay(40000, 100, 100, 400, 10)", 1),
+              ("three_bins_pay(2000, 100, 16, 48, 10)", 1), ("three_bins_pay(2000, 300, 40, 120, 10)", 1),
+              ("three_bins_pay(30000, 100, 66, 200, 10)", 1), ("three_bins_pay(2000, 300, 16, 48, 10)", 0),
+              ("three_bins_pay(5000, 100, 24, 48, 10)", 0), ("three_bins_pay(16000, 100, 33, 100, 10)", 0),
+              ("three_bins_pay(40000, 10, 33, 100, 10)", 0), ("three_bins_pay(40000, 1, 500, 4000, 10)", 0),
+              ("three_bins_pay(300, 10, 10, 100, 10)", 0),
+              ("three_bins_pay(20000, 100, 3335, 10006, 12)", 1), ("three_bins_pay(16000, 30, 133, 400, 6)", 1),
+              ("three_bins_pay(8000, 3, 66, 200, 6)", 1), ("three_bins_pay(1000, 3, 66, 200, 2)", 1),
+              ("three_bins_pay(8000, 100, 66, 200, 2)", 1), ("three_bins_pay(16000, 100, 133, 400, 4)", 1),
+              ("three_bins_pay(70000, 30, 133, 400, 10)", 1), ("three_bins_pay(70709, 31, 100, 302, 4)", 0),
+              ("three_bins_pay(103679, 14, 64, 194, 4)", 0), ("three_bins_pay(8000, 10, 400, 1200, 4)", 0),
+              ("three_bins_pay(16000, 3, 400, 1200, 6)", 0), ("three_bins_pay(70000, 3, 66, 200, 8)", 0)]
 
 
 def test_three_bins(tmp_path):
